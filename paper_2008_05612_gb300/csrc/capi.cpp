@@ -99,6 +99,8 @@ extern "C" void hp_structs_free(hp_structs* s) {
       if (t->scan_mcnt) cudaFree(t->scan_mcnt);
       if (t->scan_mmask) cudaFree(t->scan_mmask);
       if (t->scan_midx) cudaFree(t->scan_midx);
+      if (t->tc_tab) cudaFree(t->tc_tab);
+      if (t->tc_pairs) cudaFree(t->tc_pairs);
       if (t->class_first) cudaFree(t->class_first);
       if (t->class_nconf) cudaFree(t->class_nconf);
       if (t->half_otab) cudaFree(t->half_otab);

@@ -35,6 +35,10 @@ struct DevTables {
   uint32_t* scan_mmask = nullptr;  // NE x spad: per member its contact masks, word-major
   int32_t* scan_midx = nullptr;    // spad: original conformation index of each member
   int scan_ngroups = 0, scan_gpad = 0, scan_spad = 0, scan_cpad = 0;
+  // tensor-core scan (built on first use): 0/1 contact rows over the pairs that occur, in slab order
+  uint8_t* tc_tab = nullptr;
+  uint16_t* tc_pairs = nullptr;    // 32 tc_nk pairs: even index | odd index << 8
+  int tc_nk = 0, tc_ntiles = 0;    // slabs of 32 pairs (0: not built, -1: no room), tiles of 256
   // class -> first conformation index and number of conformations (built on first use)
   int32_t* class_first = nullptr;
   int32_t* class_nconf = nullptr;
@@ -81,6 +85,22 @@ namespace hp {
 int device_tables(const hp_structs* s, DevTables** out);
 // Same, plus the per-sequence scan tables.
 int scan_tables(const hp_structs* s, DevTables** out);
+// n sequences (ids, or base + row where ids is NULL) against every conformation on the tensor cores:
+// phenotypes at threshold T, and where wanted the lowest minimiser's class, the gap E2 - E1 (at most
+// T with prune) and n * S_dir added to counters[0].  err (or NULL): set to 1 on the device when a
+// wait gave up (the results are exact all the same).  Returns once enqueued; *done is the number of
+// sequences taken (0 where the tables or the scratch do not fit: not an error).
+struct ScanTc {
+  const unsigned long long* ids;
+  unsigned long long base;
+  long long n;
+  int T;
+  bool prune;
+  int32_t *phen, *aux, *gap;
+  uint64_t* counters;
+  unsigned* err;
+};
+int scan_tc(const hp_structs* s, const ScanTc& a, cudaStream_t st, long long* done);
 // Same, plus the table of reversal-canonical odd patterns (odd N).
 int half_tables(const hp_structs* s, DevTables** out);
 // Records are padded on the device to a multiple of this many conformations.
