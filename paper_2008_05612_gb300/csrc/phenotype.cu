@@ -44,6 +44,7 @@
 #include <cuda_runtime.h>
 
 #include <algorithm>
+#include <cmath>
 #include <cstdio>
 #include <cstdlib>
 #include <new>
@@ -1083,6 +1084,119 @@ int run_phenotype(const hp_structs* const* libs, const uint64_t* begins, const u
   return rc;
 }
 
+namespace {
+
+// The ids of [begin, begin + count) that the map kernel takes (the rest, on either side, go to the
+// tensor-core scan).  The map kernel shares a conformation's coefficients between all even patterns of an
+// odd one, which pays where an aligned block leaves many even residues free: a block of 2^m ids has
+// ceil(m / 2), and a CTA always evaluates 2^roles patterns.  The aligned blocks of a range grow and
+// then shrink, so the blocks of at least 2^m ids are one run; the m with the least estimated time is
+// taken.  Rates measured on 3x3x3, 2x3x4, 6x6 (scores/s): map kernel 3.5e13 with 14 roles, 3.2e13 and 3.0e13
+// with 13 and 12, 1.55e13 with 11; scan 1 / (7.9e-14 s max(1, pairs / 150) conformations + 0.62 ns) per id.
+void split_range(const hp_structs* s, uint64_t begin, uint64_t count, int gap_threshold, uint64_t* map_begin,
+                 uint64_t* map_end) {
+  constexpr double kSms = 152;
+  struct Block {
+    uint64_t at;
+    int m;
+  };
+  std::vector<Block> blocks;
+  const uint64_t end = begin + count;
+  for (uint64_t pos = begin; pos < end;) {
+    int m = 0;
+    while (m < 62 && (pos & ((2ull << m) - 1)) == 0 && pos + (2ull << m) <= end) m++;
+    blocks.push_back({pos, m});
+    pos += 1ull << m;
+  }
+  const double pairs = (double)s->NE * s->NO - (s->N - 1);  // pairs that may be in contact
+  const double scan_id = 0.62e-9 + 7.9e-14 * std::max(1.0, pairs / 150.0) * s->S_dir;
+  double best = 25e-6 + count * scan_id;  // no block to the map kernel
+  *map_begin = *map_end = begin;
+  for (int mmin = 0; mmin < 63; mmin++) {
+    uint64_t lo = end, hi = end, ids = 0;
+    int max_ne = 0;
+    for (const Block& b : blocks)
+      if (b.m >= mmin) {
+        if (lo == end) lo = b.at;
+        hi = b.at + (1ull << b.m);
+        ids += 1ull << b.m;
+        max_ne = std::max(max_ne, std::min((b.m + 1) / 2, s->NE));
+      }
+    if (!ids) break;
+    int roles = kRoles, r = 0, t = 0;
+    if (gap_threshold == 1) small_roles_shape(max_ne, &roles, &r, &t);
+    double items = 0;
+    for (const Block& b : blocks)
+      if (b.m >= mmin) {
+        const bool half = b.m == s->N && (s->N & 1) && half_enumeration_enabled();
+        const int ne = std::min((b.m + 1) / 2, s->NE);
+        items += std::ldexp(half ? 0.51 : 1.0, b.m - std::min(ne, roles));
+      }
+    const double ctas = roles == 14 ? 1 : roles == 13 ? 2 : roles == 12 ? 2 : 4;
+    const double rate = roles == 14 ? 3.5e13 : roles == 13 ? 3.2e13 : roles == 12 ? 3.0e13 : 1.55e13;
+    const double item = std::ldexp((double)s->S_dir, roles) * kSms * ctas / rate + 20e-6;
+    const double waves = std::max(1.0, items / (kSms * ctas));
+    const uint64_t rest = count - ids;
+    const double cost = 25e-6 + waves * item + (rest ? 25e-6 + rest * scan_id : 0.0);
+    if (cost < best) {
+      best = cost;
+      *map_begin = lo;
+      *map_end = hi;
+    }
+  }
+}
+
+// Ids [begin, begin + count) by the tensor-core scan; *done false where it cannot take them.
+int scan_range(const hp_structs* s, uint64_t begin, uint64_t count, int gap_threshold, int32_t* d_phen, int32_t* d_aux,
+               unsigned* err, cudaStream_t st, bool* done) {
+  *done = true;
+  if (!count) return HP_OK;
+  const ScanTc a{nullptr, begin, (long long)count, gap_threshold, false, d_phen, d_aux, nullptr, nullptr, err};
+  long long n = 0;
+  const int rc = scan_tc(s, a, st, &n);
+  *done = n == (long long)count;
+  return rc;
+}
+
+// A map of one box with no shape set on its library: split between the map kernel and the scan.
+int run_split(const hp_structs* s, uint64_t begin, uint64_t count, int gap_threshold, int32_t* d_phen, int32_t* d_aux,
+              cudaStream_t st) {
+  int r = 0, t = 0;
+  default_tile_cfg(&r, &t);
+  uint64_t b = begin, e = begin + count;
+  if (s->S < 0xFFFF) split_range(s, begin, count, gap_threshold, &b, &e);
+  if (b != begin || e != begin + count) {
+    unsigned* err = nullptr;
+    cudaError_t ce = cudaMallocAsync(&err, sizeof(unsigned), st);
+    if (ce != cudaSuccess) return cuda_fail(ce, "cudaMallocAsync(error word)");
+    cudaMemsetAsync(err, 0, sizeof(unsigned), st);
+    bool done = false;
+    int rc = scan_range(s, begin, b - begin, gap_threshold, d_phen, d_aux, err, st, &done);
+    if (rc == HP_OK && done)
+      rc = scan_range(s, e, begin + count - e, gap_threshold, d_phen + (e - begin), d_aux ? d_aux + (e - begin) : nullptr,
+                      err, st, &done);
+    unsigned herr = 0;
+    if (rc == HP_OK && done) {
+      if (e > b) {
+        int32_t *ph = d_phen + (b - begin), *ax = d_aux ? d_aux + (b - begin) : nullptr;
+        const uint64_t n = e - b;
+        rc = run_phenotype(&s, &b, &n, 1, &ph, ax ? &ax : nullptr, r, t, st, 0, gap_threshold, true);
+      }
+      if (rc == HP_OK) {
+        ce = cudaMemcpyAsync(&herr, err, sizeof(unsigned), cudaMemcpyDeviceToHost, st);
+        if (ce == cudaSuccess) ce = cudaStreamSynchronize(st);
+        if (ce != cudaSuccess) rc = cuda_fail(ce, "tensor-core scan execution");
+      }
+    }
+    cudaFreeAsync(err, st);
+    if (rc == HP_OK && herr) rc = fail(HP_ETIMEOUT, "tensor-core scan: a bounded wait timed out");
+    if (rc != HP_OK || done) return rc;
+  }
+  return run_phenotype(&s, &begin, &count, 1, &d_phen, d_aux ? &d_aux : nullptr, r, t, st, 0, gap_threshold, true);
+}
+
+}  // namespace
+
 }  // namespace hp
 
 extern "C" int hp_phenotype_map(const hp_structs* s, uint64_t seq_begin, uint64_t seq_count, int32_t gap_threshold,
@@ -1096,9 +1210,8 @@ extern "C" int hp_phenotype_map(const hp_structs* s, uint64_t seq_begin, uint64_
   const unsigned long long space = 1ull << s->N;
   if (seq_begin >= space || seq_count > space - seq_begin)
     return hp::fail(HP_EINVAL, "hp_phenotype_map: sequence range exceeds 2^N");
-  int r = s->tile_reg_bits, t = s->tile_size;
-  const bool auto_roles = r == 0;  // no shape set on the library: pick the role count from the range
-  if (!r) hp::default_tile_cfg(&r, &t);
-  return hp::run_phenotype(&s, &seq_begin, &seq_count, 1, &d_phen, d_argmin_aux ? &d_argmin_aux : nullptr, r, t,
-                           (cudaStream_t)stream, 0, gap_threshold, auto_roles);
+  if (!s->tile_reg_bits)
+    return hp::run_split(s, seq_begin, seq_count, gap_threshold, d_phen, d_argmin_aux, (cudaStream_t)stream);
+  return hp::run_phenotype(&s, &seq_begin, &seq_count, 1, &d_phen, d_argmin_aux ? &d_argmin_aux : nullptr, s->tile_reg_bits,
+                           s->tile_size, (cudaStream_t)stream, 0, gap_threshold, false);
 }

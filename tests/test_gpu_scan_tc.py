@@ -90,3 +90,17 @@ def test_exact_when_waits_give_up_and_under_capture(hp):
     graph.replay()
     graph.replay()
     assert all(torch.equal(a, b) for a, b in zip(out, want))
+
+
+@pytest.mark.parametrize("dims,begin,count,T", [((3, 3, 3), 12345, 150001, 1), ((3, 3, 3), (1 << 26) - 3, 7, 1),
+                                                ((3, 3, 3), (1 << 22) + 1, (1 << 22) + 77, 1), ((3, 3, 3), 0, 1 << 14, 9),
+                                                ((2, 3, 4), 777, 65535, 12), ((5, 5), 3, (1 << 20) + 9, 4),
+                                                ((6, 6), (1 << 35) + 5, 4097, 2), ((4, 5), 0, 1 << 20, 1)])
+def test_split_ranges_equal_the_map_kernel(hp, dims, begin, count, T):
+    """A range split between the scan and the map kernel against the map kernel alone (a library with a shape set)."""
+    s, k = hp.Structs(dims), hp.Structs(dims)
+    k.set_tile_cfg(5, 256)
+    out = [torch.full((count + 2,), -9, dtype=torch.int32, device="cuda") for _ in range(4)]
+    hp.phenotype_map(s, begin, count, out=out[0][1:-1], aux=out[1][1:-1], gap_threshold=T)
+    hp.phenotype_map(k, begin, count, out=out[2][1:-1], aux=out[3][1:-1], gap_threshold=T)
+    assert torch.equal(out[0], out[2]) and torch.equal(out[1], out[3])
