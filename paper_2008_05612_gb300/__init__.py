@@ -449,7 +449,8 @@ def phi_matrix(phen, N: int, S: int, cap: int | None = None, stream=None):
 
     if phen.numel() != (1 << N):
         raise ValueError("the phi matrix needs the full map of 2^N sequences")
-    cap = int(cap or max(1 << 16, 8 * (S + 1)))
+    # 3x3x3 has 14 to 18 entries a row; no map has more than one per flip, the diagonal and the -1 row and column
+    cap = int(cap or min(max(1 << 16, 24 * (S + 1)), (N << N) + 3 * S + 1))
     pp = _dptr(phen, torch.int32, "phen")
     row_ptr = torch.empty(S + 2, dtype=torch.int64, device=phen.device)
     while True:

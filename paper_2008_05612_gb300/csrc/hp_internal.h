@@ -108,8 +108,17 @@ constexpr int kRecPad = 256;
 // Poll limit for the bounded device-side waits of the kernels: `dflt` (the kernel's own
 // constant) unless hp_set_wait_limit has set a limit for this process.
 long long wait_limit(long long dflt);
+// Open-addressing table of the flips between two different folding phenotypes: key q << 16 | p.
+struct PhiTable {
+  uint32_t* keys;               // 2^log2cap slots, 0xFFFFFFFF where empty
+  unsigned long long* counts;
+  int log2cap;
+};
+constexpr unsigned kErrPhiFull = 16u;  // error bit: the table is full
 // Eq. 2 numerators of a full 2^N map (robustness tile pass): ADDS to neutral / to_del [S + 1] and
-// counts the -1 genotypes into *negcount (all caller-zeroed); error bits go to *err.
+// counts the -1 genotypes into *negcount (all caller-zeroed); error bits go to *err.  With phi, the
+// same passes also count into the table (S < 65535).
 cudaError_t launch_robustness(const int32_t* d_phen, int N, int S, unsigned long long* neutral,
-                              unsigned long long* to_del, unsigned long long* negcount, unsigned* err, cudaStream_t st);
+                              unsigned long long* to_del, unsigned long long* negcount, unsigned* err, cudaStream_t st,
+                              const PhiTable* phi = nullptr);
 }  // namespace hp

@@ -17,8 +17,8 @@ namespace {
 constexpr unsigned kErrRange = 4u;     // a map entry outside [-1, S)
 constexpr unsigned kErrUnion = 8u;     // union retries exhausted
 constexpr int kHistThreads = 1024;
-constexpr int kRobTileBits = 13;       // 2^13 ids (32 KB) of the map per block, two blocks per CTA
-constexpr int kRobMaxPassBits = 8;     // high bits per later pass (a block keeps >= 32 contiguous ids)
+constexpr int kRobTileBits = 13;       // up to 2^13 ids (32 KB) of the map per block, two blocks per CTA
+constexpr int kRobMaxPassBits = 8;     // high bits per later pass (a block of 2^13 keeps >= 32 contiguous ids)
 constexpr int kRobThreads = 512;
 constexpr int kRobReplicas = 16;       // copies of each phenotype's two counters (spreads hot-phenotype atomics)
 
@@ -81,6 +81,7 @@ __global__ void hist_sum(const unsigned* __restrict__ partial, int rows, int S, 
   const int b = blockIdx.x * blockDim.x + threadIdx.x;
   if (b > S) return;
   unsigned long long s = accumulate ? hist[b] : 0ull;
+#pragma unroll 8
   for (int r = 0; r < rows; r++) s += partial[(size_t)r * (S + 1) + b];
   hist[b] = s;
 }
@@ -120,7 +121,55 @@ __global__ void hist_global(const int32_t* __restrict__ phen, unsigned long long
   if ((threadIdx.x & 31) == 0 && neg) atomicAdd(&hist[S], (unsigned long long)neg);
 }
 
-// ---------------------------------------------------------------- robustness
+// ---------------------------------------------------------------- unions (components)
+
+// Root of x: parents always have smaller ids, so the walk terminates.
+__device__ __forceinline__ int32_t cc_root(const int32_t* label, int32_t x) {
+  int32_t par = __ldcg(label + x);
+  while (par != x) {
+    x = par;
+    par = __ldcg(label + x);
+  }
+  return x;
+}
+
+// Lock-free union of the components of a and b (Rem's algorithm with compare-and-swap splicing): the two
+// walks go up together, their parents loaded side by side; the side with the larger parent moves, its
+// node spliced under the other's parent on the way, until the parents agree or a root is hooked.
+// Parents only decrease, so the roots are the components' smallest ids, and a failed CAS means another
+// thread moved that node on.  Bounded all the same (false if it gives up).  T: ids in global memory, or local
+// indices of a block in shared memory.
+template <class T>
+__device__ __forceinline__ bool join(T* label, T a, T b) {
+  volatile T* l = label;
+  T pa = l[a], pb = l[b];
+  for (int tries = 0; tries < (1 << 26); tries++) {
+    if (pa == pb) return true;
+    if (pa < pb) {
+      const T t = a, tp = pa;
+      a = b;
+      pa = pb;
+      b = t;
+      pb = tp;
+    }
+    const T seen = atomicCAS(label + a, pa, pb);
+    if (a == pa) {
+      if (seen == pa) return true;  // a was a root: hooked
+      pa = seen;
+    } else {
+      a = pa;
+      pa = l[a];
+    }
+  }
+  return false;
+}
+
+__device__ __forceinline__ unsigned tile_root(const uint16_t* par, unsigned x) {
+  for (unsigned q = par[x]; q != x; q = par[x]) x = q;
+  return x;
+}
+
+// ---------------------------------------------------------------- passes over the flips
 
 // Eq. 2 numerators in passes over the map, each reading it once.  A block is 2^kRobTileBits ids
 // in shared memory: 2^c consecutive ids times every combination of the pass's h bits
@@ -147,12 +196,45 @@ __device__ __forceinline__ void cp_async16(void* dst, const void* src) {
                : "memory");
 }
 
-__global__ void __launch_bounds__(kRobThreads) robustness_pass(const int32_t* __restrict__ phen, int S, const RobPass P,
+__device__ __forceinline__ uint32_t phi_slot(uint32_t key, int log2cap) { return (key * 0x9E3779B1u) >> (32 - log2cap); }
+
+// Add 1 to the count of key in the table (linear probing, bounded; a table found full ends every
+// thread's probing, since the call then fails).
+__device__ __forceinline__ void phi_add(const hp::PhiTable& t, uint32_t key, unsigned* err) {
+  const uint32_t mask = (1u << t.log2cap) - 1u;
+  uint32_t s = phi_slot(key, t.log2cap);
+  for (uint32_t probe = 0; probe <= mask; probe++, s = (s + 1) & mask) {
+    uint32_t k = t.keys[s];
+    if (k == 0xFFFFFFFFu) {
+      k = atomicCAS(t.keys + s, 0xFFFFFFFFu, key);
+      if (k == 0xFFFFFFFFu) k = key;
+    }
+    if (k == key) {
+      atomicAdd(t.counts + s, 1ull);
+      return;
+    }
+    if ((probe & 255u) == 255u && (*reinterpret_cast<volatile unsigned*>(err) & hp::kErrPhiFull)) return;
+  }
+  atomicOr(err, hp::kErrPhiFull);
+}
+
+// What a pass does with the flips: the Eq. 2 numerators; these and the phi table (flips to another folding
+// phenotype); or the unions of the neutral networks.  For the networks the first pass joins each block of
+// 2^13 ids by a union-find in shared memory and writes the block's labels (-1 where the id does not fold),
+// and the later passes join ids across the pass's bits through the labels in global memory, comparing
+// phenotypes in shared memory.  2^25 ids at the 3x3x3 density: 200 + 286 us and 84 us for the last walk (the
+// unions wait on dependent reads), where one pass that read every partner from global memory and joined
+// all flips through global labels took 67 + 566 + 178 us.
+enum FlipWork { kRobustness, kPhi, kJoinFirst, kJoin };
+
+template <int WORK>
+__global__ void __launch_bounds__(kRobThreads) flip_pass(const int32_t* __restrict__ phen, int S, const RobPass P,
                                                                unsigned long long nblocks, int replicas,
                                                                unsigned long long* __restrict__ neutral_rep,
                                                                unsigned long long* __restrict__ to_del_rep,
                                                                unsigned long long* __restrict__ negcount,
-                                                               unsigned* __restrict__ err) {
+                                                               unsigned* __restrict__ err, const hp::PhiTable phi, int32_t* label) {
+  constexpr bool PHI = WORK == kPhi;
   extern __shared__ int32_t tiles[];  // two blocks, then the list of a block's genotypes that fold
   __shared__ unsigned long long hoff[1 << kRobMaxPassBits];
   __shared__ unsigned nlist;
@@ -193,6 +275,28 @@ __global__ void __launch_bounds__(kRobThreads) robustness_pass(const int32_t* __
   unsigned long long* __restrict__ neutral = neutral_rep + (size_t)(blockIdx.x % replicas) * S;
   unsigned long long* __restrict__ to_del = to_del_rep + (size_t)(blockIdx.x % replicas) * S;
   unsigned neg = 0;
+  // networks: this warp's pairs to join, and joining up to 32 of them
+  __shared__ uint2 pair_buf[WORK >= kJoinFirst ? kRobThreads / 32 : 1][WORK == kJoinFirst ? 64 : 128];
+  uint2* pairs = pair_buf[WORK >= kJoinFirst ? threadIdx.x >> 5 : 0];
+  int pending = 0;
+  auto join_pairs = [&] {
+    pending = max(pending - 32, 0);  // the newest ones
+    const uint2 q = pairs[pending + lane];
+    if (q.x != ~0u && !(WORK == kJoinFirst ? join<unsigned short>(list + kIds, (unsigned short)q.x, (unsigned short)q.y)
+                                           : join<int>(label, (int)q.x, (int)q.y)))
+      atomicOr(err, kErrUnion);
+    __syncwarp();
+  };
+  auto join_rest = [&] {
+    while (pending) {
+      if (pending < 32) {  // fill the round with empty pairs
+        if (lane >= pending) pairs[lane] = make_uint2(~0u, ~0u);
+        __syncwarp();
+        pending = 32;
+      }
+      join_pairs();
+    }
+  };
   unsigned long long b = blockIdx.x;
   if (vec && b < nblocks) issue(b, 0);
   for (int it = 0; b < nblocks; b += gridDim.x, it++) {
@@ -252,7 +356,50 @@ __global__ void __launch_bounds__(kRobThreads) robustness_pass(const int32_t* __
     }
     __syncthreads();
     // phase 2: one listed genotype per lane, its counted flips in turn
-    {
+    if constexpr (WORK == kJoinFirst || WORK == kJoin) {
+      const unsigned n = nlist;
+      const unsigned long long base = block_base(b);
+      uint16_t* par = list + kIds;
+      if (WORK == kJoinFirst) {
+        for (unsigned f = threadIdx.x; f < n; f += blockDim.x) par[list[f]] = list[f];
+        __syncthreads();
+      }
+      // One id in ten or so has a partner to join at a bit, and a union is a chain of dependent reads, so
+      // each warp collects its pairs and joins 32 at a time.  In shared memory the pairs are of this
+      // block; across blocks they are global ids and wait for the warp's next ones.
+      const uint32_t lt = (1u << lane) - 1u;
+      for (unsigned f0 = threadIdx.x - lane; f0 < n; f0 += blockDim.x) {
+        const bool have = f0 + lane < n;
+        const unsigned idx = have ? list[f0 + lane] : 0u;
+        const int32_t p = tile[idx];
+        const uint32_t id = WORK == kJoinFirst ? idx : (uint32_t)(base + hoff[idx >> c] + (idx & cmask));
+        for (int t = 0; t < nbits; t++) {
+          const unsigned other = idx ^ (1u << (bit0 + t));
+          const bool hit = have && other > idx && tile[other] == p;  // each pair once, from its smaller id
+          const uint32_t m = __ballot_sync(0xFFFFFFFFu, hit);
+          if (!m) continue;
+          if (hit) pairs[pending + __popc(m & lt)] = make_uint2(id, WORK == kJoinFirst ? other : id | (1u << P.pos[t]));
+          pending += __popc(m);
+          __syncwarp();
+          if (pending >= (WORK == kJoinFirst ? 32 : 96)) join_pairs();
+        }
+      }
+      // the warps of a CTA join their waiting pairs at the same blocks (a block waits for the slowest
+      // warp's union, several dependent reads of global memory)
+      if (WORK == kJoinFirst || (it & 3) == 3) join_rest();
+      if (WORK == kJoinFirst) {
+        __syncthreads();
+        auto root = [&](unsigned j) {
+          return (unsigned)tile[j] < (unsigned)S ? (int32_t)(base + tile_root(par, j)) : -1;
+        };
+        if (vec && reinterpret_cast<uintptr_t>(label) % 16 == 0) {
+          for (unsigned j = 4 * threadIdx.x; j < ids; j += 4 * blockDim.x)
+            *reinterpret_cast<int4*>(label + base + j) = make_int4(root(j), root(j + 1), root(j + 2), root(j + 3));
+        } else {
+          for (unsigned j = threadIdx.x; j < ids; j += blockDim.x) label[base + j] = root(j);
+        }
+      }
+    } else {
       const unsigned n = nlist;
       for (unsigned f = threadIdx.x; f < n; f += blockDim.x) {
         const unsigned idx = list[f];
@@ -262,6 +409,7 @@ __global__ void __launch_bounds__(kRobThreads) robustness_pass(const int32_t* __
           const int32_t q = tile[idx ^ (1u << (bit0 + t))];
           nn += q == p;
           nd += q < 0;
+          if (PHI && q >= 0 && q != p && q < S) phi_add(phi, ((uint32_t)p << 16) | (uint32_t)q, err);
         }
         if (nn) atomicAdd(&neutral[p], (unsigned long long)nn);
         if (nd) atomicAdd(&to_del[p], (unsigned long long)nd);
@@ -269,25 +417,41 @@ __global__ void __launch_bounds__(kRobThreads) robustness_pass(const int32_t* __
     }
     __syncthreads();  // the slot is refilled by the copy issued in the next iteration but one
   }
-  if (P.first) {
+  if (WORK == kJoin) join_rest();
+  if (P.first && negcount) {
     for (int off = 16; off; off >>= 1) neg += __shfl_xor_sync(0xFFFFFFFFu, neg, off);
     if (lane == 0 && neg) atomicAdd(negcount, (unsigned long long)neg);
   }
 }
 
-__global__ void robustness_gather(const unsigned long long* __restrict__ rep, int replicas, int S,
-                                  unsigned long long* __restrict__ neutral, unsigned long long* __restrict__ to_del) {
+// Sums of the replicas, and with the last block's ticket the -1 entry by the edge identity (a launch of
+// one CTA for it walked 51,704 counters in 25 us).  tail: [sum of to_del][blocks done], zeroed.
+__global__ void robustness_gather(const unsigned long long* __restrict__ rep, int replicas, int N, int S,
+                                  unsigned long long* __restrict__ neutral, unsigned long long* __restrict__ to_del,
+                                  const unsigned long long* __restrict__ negcount, unsigned long long* tail) {
   const int p = blockIdx.x * blockDim.x + threadIdx.x;
-  if (p >= S) return;
   unsigned long long a = 0, d = 0;
-  for (int r = 0; r < replicas; r++) {
-    a += rep[(size_t)r * S + p];
-    d += rep[(size_t)(replicas + r) * S + p];
+  if (p < S) {
+#pragma unroll 8
+    for (int r = 0; r < replicas; r++) {
+      a += rep[(size_t)r * S + p];
+      d += rep[(size_t)(replicas + r) * S + p];
+    }
+    neutral[p] = a;
+    to_del[p] = d;
   }
-  neutral[p] = a;
-  to_del[p] = d;
+  for (int off = 16; off; off >>= 1) d += __shfl_xor_sync(0xFFFFFFFFu, d, off);
+  if ((threadIdx.x & 31) == 0 && d) atomicAdd(tail, d);
+  __threadfence();
+  __syncthreads();
+  if (threadIdx.x == 0 && atomicAdd(tail + 1, 1ull) == gridDim.x - 1) {
+    const unsigned long long v = (unsigned long long)N * negcount[0] - atomicAdd(tail, 0ull);
+    neutral[S] = v;
+    to_del[S] = v;
+  }
 }
 
+// The -1 entry where there are no replicas.
 __global__ void robustness_finish(int N, int S, unsigned long long* __restrict__ neutral,
                                   unsigned long long* __restrict__ to_del, const unsigned long long* __restrict__ negcount) {
   __shared__ unsigned long long part[32];
@@ -307,89 +471,29 @@ __global__ void robustness_finish(int N, int S, unsigned long long* __restrict__
 
 // ---------------------------------------------------------------- components
 
-__global__ void cc_init(const int32_t* __restrict__ phen, unsigned long long total, int S, int32_t* __restrict__ label,
-                        unsigned* __restrict__ err) {
-  const unsigned long long stride = (unsigned long long)gridDim.x * blockDim.x;
-  for (unsigned long long g = (unsigned long long)blockIdx.x * blockDim.x + threadIdx.x; g < total; g += stride) {
-    const int32_t p = phen[g];
-    if (p < -1 || p >= S) atomicOr(err, kErrRange);
-    label[g] = (p >= 0 && p < S) ? (int32_t)g : -1;
-  }
-}
-
-// Root of x: parents always have smaller ids, so the walk terminates.
-__device__ __forceinline__ int32_t cc_root(const int32_t* label, int32_t x) {
-  int32_t par = __ldcg(label + x);
-  while (par != x) {
-    x = par;
-    par = __ldcg(label + x);
-  }
-  return x;
-}
-
-// The same with path halving, while components are being joined: each visited id is pointed at
-// its grandparent (an ancestor with a smaller id, so concurrent finds and hooks stay correct;
-// hooks only change roots, which are never rewritten).  Not for the final compression, where a
-// late halving write could replace an id's final root by a non-root ancestor.
-__device__ __forceinline__ int32_t cc_find(int32_t* label, int32_t x) {
-  for (;;) {
-    const int32_t q = __ldcg(label + x);
-    if (q == x) return x;
-    const int32_t g = __ldcg(label + q);
-    if (g == q) return q;
-    __stcg(label + x, g);
-    x = g;
-  }
-}
-
-// Lock-free union of the components of a and b: hook the larger root under the smaller one with
-// a CAS and retry from the value the CAS saw.  Every failed CAS means another thread linked that
-// root, so the loop makes progress; it is bounded all the same (false if it gives up).
-__device__ __forceinline__ bool cc_union(int32_t* label, int32_t a, int32_t b) {
-  for (int tries = 0; tries < (1 << 24); tries++) {
-    const int32_t ra = cc_find(label, a), rb = cc_find(label, b);
-    if (ra == rb) return true;
-    const int32_t lo = min(ra, rb), hi = max(ra, rb);
-    const int32_t seen = atomicCAS(label + hi, hi, lo);
-    if (seen == hi) return true;
-    a = lo;
-    b = seen;
-  }
-  return false;
-}
-
-// One warp per 32 consecutive ids: the (id, flipped bit) pairs of its non-deleterious ids are
-// spread over the lanes (about 1.5 such ids per 32 in 3x3x3), so the partner reads and unions of
-// different pairs are in flight together instead of one lane walking all N bits.
-__global__ void cc_hook(const int32_t* __restrict__ phen, int N, int32_t* label, unsigned* __restrict__ err) {
-  const unsigned long long total = 1ull << N;
-  const int lane = threadIdx.x & 31;
-  const unsigned long long warps = (unsigned long long)gridDim.x * (blockDim.x >> 5);
-  for (unsigned long long base = ((unsigned long long)blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5)) * 32;
-       base < total; base += warps * 32) {
-    const unsigned long long g = base + lane;
-    const bool fold = g < total && __ldcg(label + g) >= 0;  // deleterious ids carry label -1
-    const uint32_t bal = __ballot_sync(0xFFFFFFFFu, fold);
-    const int npairs = __popc(bal) * N;
-    for (int k = lane; k < npairs; k += 32) {
-      const int src = __fns(bal, 0, k / N + 1), i = k % N;
-      const unsigned long long gs = base + src, h = gs ^ (1ull << i);
-      if (h < gs) continue;  // each pair once, from its smaller id
-      if (__ldg(phen + h) != __ldg(phen + gs)) continue;
-      if (!cc_union(label, (int32_t)gs, (int32_t)h)) atomicOr(err, kErrUnion);
-    }
-  }
-}
-
+// Every label to its root, and a component counted at each root; four ids of a thread at a time (their
+// walks in flight together).
 __global__ void cc_finish(const int32_t* __restrict__ phen, unsigned long long total, int32_t* label,
                           unsigned long long* __restrict__ ncomp) {
-  const unsigned long long stride = (unsigned long long)gridDim.x * blockDim.x;
-  for (unsigned long long g = (unsigned long long)blockIdx.x * blockDim.x + threadIdx.x; g < total; g += stride) {
-    const int32_t l = label[g];
-    if (l < 0) continue;
-    const int32_t r = cc_root(label, (int32_t)g);
-    label[g] = r;
-    if (r == (int32_t)g) atomicAdd(&ncomp[phen[g]], 1ull);
+  const unsigned long long stride = 4ull * gridDim.x * blockDim.x;
+  const bool vec = reinterpret_cast<uintptr_t>(label) % 16 == 0;
+  for (unsigned long long g = 4ull * ((unsigned long long)blockIdx.x * blockDim.x + threadIdx.x); g < total; g += stride) {
+    int32_t l[4] = {-1, -1, -1, -1};
+    if (vec && g + 3 < total) {
+      const int4 q = *reinterpret_cast<const int4*>(label + g);
+      l[0] = q.x; l[1] = q.y; l[2] = q.z; l[3] = q.w;
+    } else {
+#pragma unroll
+      for (int k = 0; k < 4; k++)
+        if (g + k < total) l[k] = label[g + k];
+    }
+#pragma unroll
+    for (int k = 0; k < 4; k++) {
+      if (l[k] < 0) continue;
+      const int32_t r = cc_root(label, l[k]);
+      if (r != l[k]) label[g + k] = r;
+      if (r == (int32_t)(g + k)) atomicAdd(&ncomp[phen[g + k]], 1ull);
+    }
   }
 }
 
@@ -477,11 +581,16 @@ extern "C" int hp_robustness(const int32_t* d_phen, int32_t N, int32_t S, uint64
 
 namespace hp {
 
+// Ids per block: 2^13, or fewer for small maps, so that they still have 2^7 blocks or so to spread over
+// the SMs and one later pass (4x4, 2^16 ids: Eq. 2 passes 20 -> 12 us,
+// networks 41 + 25 -> 10 + 18 us, against blocks of 2^13).
+int flip_block_bits(int N) { return std::min(N, std::max(9, std::min(kRobTileBits, N - 8))); }
+
 // The passes over the flips of an N-bit map: bits [0, k) first, then the high bits [k, N) in
-// near-equal groups of at most kRobMaxPassBits, each with the kRobTileBits - h lowest bits
-// contiguous (k = min(N, kRobTileBits)).
+// near-equal groups of at most kRobMaxPassBits, each with the k - h lowest bits
+// contiguous.
 std::vector<RobPass> flip_passes(int N) {
-  const int k = std::min((int)N, kRobTileBits);
+  const int k = flip_block_bits(N);
   std::vector<RobPass> plan;
   {
     RobPass p{};
@@ -496,7 +605,7 @@ std::vector<RobPass> flip_passes(int N) {
   for (int i = 0, lo = k; i < np; i++) {
     RobPass p{};
     p.h = R / np + (i < R % np ? 1 : 0);
-    p.c = kRobTileBits - p.h;
+    p.c = k - p.h;
     for (int t = 0; t < p.h; t++) p.pos[t] = lo + t;
     for (int b = p.c; b < N; b++)
       if (b < lo || b >= lo + p.h) p.rest[p.nrest++] = b;
@@ -507,18 +616,20 @@ std::vector<RobPass> flip_passes(int N) {
 }
 
 cudaError_t launch_robustness(const int32_t* d_phen, int N, int S, unsigned long long* neutral,
-                              unsigned long long* to_del, unsigned long long* negcount, unsigned* err, cudaStream_t st) {
-  const int k = std::min((int)N, kRobTileBits);
-  const unsigned long long blocks = 1ull << (N - k);
+                              unsigned long long* to_del, unsigned long long* negcount, unsigned* err, cudaStream_t st,
+                              const PhiTable* phi) {
+  const unsigned long long blocks = 1ull << (N - flip_block_bits(N));
   const size_t smem = 2 * (sizeof(int32_t) << kRobTileBits) + (sizeof(uint16_t) << kRobTileBits);
-  cudaError_t e = cudaFuncSetAttribute(robustness_pass, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+  const auto pass = phi ? flip_pass<kPhi> : flip_pass<kRobustness>;
+  const PhiTable table = phi ? *phi : PhiTable{};
+  cudaError_t e = cudaFuncSetAttribute(pass, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
   if (e != cudaSuccess) return e;
   const std::vector<RobPass> plan = flip_passes(N);
   // a few CTAs per SM walking the blocks (shared memory: two blocks each), counting into
   // replicated counters (stream-ordered scratch; without it, straight into neutral / to_del)
   const unsigned grid = (unsigned)std::min<unsigned long long>(blocks, (unsigned long long)sm_count() * 2);
   unsigned long long* rep = nullptr;
-  const size_t rep_bytes = sizeof(unsigned long long) * 2 * kRobReplicas * (size_t)S;
+  const size_t rep_bytes = sizeof(unsigned long long) * (2 * kRobReplicas * (size_t)S + 2);
   if (cudaMallocAsync(&rep, rep_bytes, st) != cudaSuccess || cudaMemsetAsync(rep, 0, rep_bytes, st) != cudaSuccess) {
     if (rep) cudaFreeAsync(rep, st);
     rep = nullptr;
@@ -526,16 +637,18 @@ cudaError_t launch_robustness(const int32_t* d_phen, int N, int S, unsigned long
   }
   for (const RobPass& p : plan) {
     if (rep)
-      robustness_pass<<<grid, kRobThreads, smem, st>>>(d_phen, S, p, blocks, kRobReplicas, rep, rep + (size_t)kRobReplicas * S,
-                                                       negcount, err);
+      pass<<<grid, kRobThreads, smem, st>>>(d_phen, S, p, blocks, kRobReplicas, rep, rep + (size_t)kRobReplicas * S, negcount,
+                                            err, table, nullptr);
     else
-      robustness_pass<<<grid, kRobThreads, smem, st>>>(d_phen, S, p, blocks, 1, neutral, to_del, negcount, err);
+      pass<<<grid, kRobThreads, smem, st>>>(d_phen, S, p, blocks, 1, neutral, to_del, negcount, err, table, nullptr);
   }
   if (rep) {
-    robustness_gather<<<(S + 255) / 256, 256, 0, st>>>(rep, kRobReplicas, S, neutral, to_del);
+    robustness_gather<<<(S + 255) / 256, 256, 0, st>>>(rep, kRobReplicas, N, S, neutral, to_del, negcount,
+                                                       rep + 2 * kRobReplicas * (size_t)S);
     cudaFreeAsync(rep, st);
+  } else {
+    robustness_finish<<<1, 1024, 0, st>>>(N, S, neutral, to_del, negcount);
   }
-  robustness_finish<<<1, 1024, 0, st>>>(N, S, neutral, to_del, negcount);
   return cudaGetLastError();
 }
 
@@ -552,12 +665,25 @@ extern "C" int hp_neutral_components(const int32_t* d_phen, int32_t N, int32_t S
   if (e != cudaSuccess) return hp::cuda_fail(e, "hp_neutral_components: cudaMallocAsync");
   cudaMemsetAsync(err, 0, sizeof(unsigned), st);
   cudaMemsetAsync(d_ncomp, 0, sizeof(uint64_t) * (size_t)S, st);
-  const unsigned long long total = 1ull << N;
-  const unsigned grid = (unsigned)std::min<unsigned long long>((total + 255) / 256, (unsigned long long)sm_count() * 16);
-  cc_init<<<grid, 256, 0, st>>>(d_phen, total, S, d_label, err);
-  cc_hook<<<grid, 256, 0, st>>>(d_phen, N, d_label, err);
-  cc_finish<<<grid, 256, 0, st>>>(d_phen, total, d_label, reinterpret_cast<unsigned long long*>(d_ncomp));
-  e = cudaGetLastError();
+  const unsigned long long total = 1ull << N, blocks = total >> hp::flip_block_bits(N);
+  const unsigned pgrid = (unsigned)std::min<unsigned long long>(blocks, (unsigned long long)sm_count() * 2);
+  const size_t smem = 2 * (sizeof(int32_t) << kRobTileBits) + (sizeof(uint16_t) << kRobTileBits);
+  const size_t smem1 = smem + (sizeof(uint16_t) << kRobTileBits);  // and the block's parents
+  e = cudaFuncSetAttribute(flip_pass<kJoinFirst>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem1);
+  if (e == cudaSuccess) e = cudaFuncSetAttribute(flip_pass<kJoin>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+  if (e == cudaSuccess) {
+    for (const RobPass& p : hp::flip_passes(N)) {
+      if (p.first)
+        flip_pass<kJoinFirst><<<pgrid, kRobThreads, smem1, st>>>(d_phen, S, p, blocks, 1, nullptr, nullptr, nullptr, err,
+                                                                  hp::PhiTable{}, d_label);
+      else
+        flip_pass<kJoin><<<pgrid, kRobThreads, smem, st>>>(d_phen, S, p, blocks, 1, nullptr, nullptr, nullptr, err,
+                                                            hp::PhiTable{}, d_label);
+    }
+    const unsigned grid = (unsigned)std::min<unsigned long long>((total + 1023) / 1024, (unsigned long long)sm_count() * 16);
+    cc_finish<<<grid, 256, 0, st>>>(d_phen, total, d_label, reinterpret_cast<unsigned long long*>(d_ncomp));
+    e = cudaGetLastError();
+  }
   int rc = e == cudaSuccess ? HP_OK : hp::cuda_fail(e, "hp_neutral_components: launch");
   return finish_with_err(err, st, "hp_neutral_components", rc);
 }
