@@ -21,8 +21,8 @@
 // three-input maxima and five more instructions per 32 scores.
 // A unit takes 2 x 128 clk per 32 pairs at the tensor cores' rate; each half has one accumulator, so a
 // half's drain and hand-over (about 400 clk) overlap only the other half's multiplications.
-// Measured (call, ids in L2): 16,384 ids of 3x3x3 182 us, the warp scan 13,600 us; 65,536 ids of 6x6
-// 700 us, the pruned warp scan 6,400 us; floors at 128 clk per 128 x 256 x 32: 110 and 480 us.
+// Measured (call, ids in L2): 16,384 ids of 3x3x3 170 us, the warp scan 13,600 us; 65,536 ids of 6x6
+// 660 us, the pruned warp scan 6,400 us; floors at 128 clk per 128 x 256 x 32: 110 and 480 us.
 //
 // scan_tc_resolve: one warp per sequence merges the runs' results and scores the one group of 32
 // conformations exactly, which gives the lowest minimiser, the tie and the energy gap.
@@ -93,7 +93,7 @@ __device__ __forceinline__ bool poll(uint32_t bar, uint32_t parity) {
 
 // Bounded wait for a barrier phase; one that gives up raises the CTA's abort flag, which ends the
 // other roles' waits too.
-__device__ bool wait_phase(uint64_t* bar, uint32_t parity, volatile int* abort_flag, uint32_t limit) {
+__device__ __noinline__ bool wait_phase(uint64_t* bar, uint32_t parity, volatile int* abort_flag, uint32_t limit) {
   const uint32_t b = sa(bar);
   for (uint32_t i = 0;; i++) {
     if (i >= limit) {
@@ -103,6 +103,12 @@ __device__ bool wait_phase(uint64_t* bar, uint32_t parity, volatile int* abort_f
     if (poll(b, parity)) return true;
     if ((i & 255) == 255 && *abort_flag) return false;
   }
+}
+
+// The same by a converged warp for a barrier that is usually complete: one poll, then the loop.
+__device__ __forceinline__ bool warp_wait(uint64_t* bar, uint32_t parity, volatile int* abort_flag, uint32_t limit) {
+  if (limit != 0 && __all_sync(0xFFFFFFFFu, poll(sa(bar), parity))) return true;
+  return __all_sync(0xFFFFFFFFu, wait_phase(bar, parity, abort_flag, limit));
 }
 
 __device__ __forceinline__ void drain(uint64_t* bar, uint32_t parity) {
@@ -260,32 +266,32 @@ __global__ void __launch_bounds__(kThreads, 1) scan_tc_kernel(const TcParams p) 
     while (u < u1 && ok) {
       const long long blk = u / p.ntiles, uend = min(u1, (blk + 1) * p.ntiles);
       const bool mine = h == 0 || p.n - blk * kBlock > kRows;  // else: only hand the stages back
-      ok = __all_sync(0xFFFFFFFFu, wait_phase(&afull, seg & 1, abort_flag, p.spin));
+      ok = warp_wait(&afull, seg & 1, abort_flag, p.spin);
       seg++;
       for (int left = (int)(uend - u); left > 0 && ok; left--) {
         uint32_t ad = a0;
         for (int k = 0; k < nk && ok; k += p.cs) {
-          ok = __all_sync(0xFFFFFFFFu, wait_phase(&full[slot], round & 1, abort_flag, p.spin));
+          ok = warp_wait(&full[slot], round & 1, abort_flag, p.spin);
           // (after the stage: that wait then overlaps the epilogue's drain of this accumulator)
           if (k == 0 && mine && ok) {
-            ok = __all_sync(0xFFFFFFFFu, wait_phase(&tempty[h], (uses & 1) ^ 1, abort_flag, p.spin));
+            ok = warp_wait(&tempty[h], (uses & 1) ^ 1, abort_flag, p.spin);
             uses++;
           }
           if (!ok) break;
           asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
           const uint32_t bd = b0 + slot * bstage;
-          const int ke = min(p.cs, nk - k);
+          const int ke = min(p.cs, nk - k), freed = slot;
+          if (++slot == p.nslots) {
+            slot = 0;
+            round++;
+          }
           if (mine) {
 #pragma unroll
             for (int i = 0; i < kMaxStage; i++)
               if (i < ke) mma(acc, ad + i * (kSlabA >> 4), bd + i * (kSlabB >> 4), k + i > 0);
           }
           ad += ke * (kSlabA >> 4);
-          commit(&empty[slot]);
-          if (++slot == p.nslots) {
-            slot = 0;
-            round++;
-          }
+          commit(&empty[freed]);
         }
         if (ok && mine) commit(&tfull[h]);
       }
@@ -341,7 +347,7 @@ __global__ void __launch_bounds__(kThreads, 1) scan_tc_kernel(const TcParams p) 
 #pragma unroll
         for (int h = 0; h < 2; h++) {
           if (h >= halves || !ok) continue;
-          ok = __all_sync(0xFFFFFFFFu, wait_phase(&tfull[h], uses[h] & 1, abort_flag, p.spin));
+          ok = warp_wait(&tfull[h], uses[h] & 1, abort_flag, p.spin);
           if (!ok) continue;
           uses[h]++;
           asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");

@@ -3,8 +3,8 @@
 // One persistent CTA per SM walks the 128 x 256 output tiles (m fastest, so the CTAs running at
 // the same time share B tiles in L2).  Warp roles:
 //   warp 0, one lane  TMA producer: 64-wide K chunks of A (128 x 64) and B (256 x 64) into a
-//                     3-stage ring, 128-byte swizzled, completion counted on full[s];
-//   warp 1, one lane  MMA issuer: four tcgen05.mma (M 128, N 256, K 16) per chunk into one of two
+//                     3- or 4-stage ring, 128-byte swizzled, completion counted on full[s];
+//   warp 1            MMA issuer: four tcgen05.mma (M 128, N 256, K 16) per chunk into one of two
 //                     tensor-memory accumulators (2 x 256 columns), commit -> empty[s] frees the
 //                     stage, commit -> tmem_full[a] hands the finished accumulator over;
 //   warps 2..9        epilogue, two warps per lane quarter and 128 columns each: tcgen05.ld
@@ -23,7 +23,6 @@
 #include <cmath>
 #include <cstring>
 #include <mutex>
-#include <numeric>
 
 #include "hp_internal.h"
 #include "tc_gemm.h"
@@ -36,22 +35,21 @@ using bf16 = __nv_bfloat16;
 constexpr int TM = kTcTileM, TN = kTcTileN, TK = 64;
 constexpr int A_BYTES = TM * TK * 2, B_BYTES = TN * TK * 2, STAGE_BYTES = A_BYTES + B_BYTES;
 constexpr int SQ_FLOATS = 32 * 33;  // store mode: one epilogue warp's padded 32 x 32 square
-constexpr int SX_FLOATS = 32 * 32;  // top-k mode: one epilogue warp's staged logits (XOR-swizzled rows)
 // gradient mode: per epilogue warp two staging buffers, each a 32 x 32 bf16 block of dz
 // (row-major, 64-byte rows), the sources of the TMA stores
 constexpr int STG_BLOCK = 32 * 32 * 2, STG_WARP = 2 * STG_BLOCK;
 // Epilogue warps: 16, four per tensor-memory lane quarter, 64 columns each (more warps hide the
 // tensor-memory and global-memory latencies of the epilogues), except in top-k mode, which keeps
 // 8 (two per lane quarter, 128 columns each; each warp keeps one candidate list per row).  Top-k and
-// softmax modes also keep the warp's biases of the current tile in shared memory; a 3-stage ring
-// leaves room for the warps' shared-memory areas.
+// softmax modes also keep the warp's biases of the current tile in shared memory; the ring has the
+// stages that the warps' shared-memory areas leave room for.
 template <int KT>
 struct Shape {
   static constexpr int kEpiWarps = KT > 0 ? 4 * tc_topk_lists_per_tile(KT) : 16;
   static constexpr int kThreads = 64 + 32 * kEpiWarps;
   static constexpr int kColsPerWarp = TN / (kEpiWarps / 4);
-  static constexpr int kStages = 3;
-  static constexpr int kAreaFloats = KT > 0 ? SX_FLOATS + kColsPerWarp : KT < 0 ? kColsPerWarp : SQ_FLOATS;
+  static constexpr int kStages = KT > 0 || KT == -1 ? 4 : 3;
+  static constexpr int kAreaFloats = KT != 0 ? kColsPerWarp : SQ_FLOATS;
   static constexpr int kStgBytes = KT == -2 ? kEpiWarps * STG_WARP : 0;
   static constexpr int kSmem = kStages * STAGE_BYTES + kStgBytes + kEpiWarps * kAreaFloats * 4 + 1024;
 };
@@ -102,8 +100,7 @@ __device__ __forceinline__ bool poll(uint32_t bar, uint32_t parity) {
 // Wait for the phase of `bar` with this parity.  False if another role aborted (checked every
 // 256 polls) or, after `limit` polls, this one gives up (then it raises the abort flag and the
 // error word); a limit of 0 gives up before the first poll.
-__device__ bool wait_or_abort(uint64_t* bar, uint32_t parity, volatile int* abort_flag, unsigned* err, uint32_t limit) {
-  const uint32_t b = sa(bar);
+__device__ __noinline__ bool wait_or_abort(uint32_t b, uint32_t parity, volatile int* abort_flag, unsigned* err, uint32_t limit) {
   for (uint32_t i = 0;; i++) {
     if (i >= limit) {
       *abort_flag = 1;
@@ -115,6 +112,13 @@ __device__ bool wait_or_abort(uint64_t* bar, uint32_t parity, volatile int* abor
   }
 }
 
+// The same by a converged warp for a barrier that is usually complete: one poll, then the loop.
+__device__ __forceinline__ bool warp_wait(uint32_t bar, uint32_t parity, volatile int* abort_flag, unsigned* err,
+                                          uint32_t limit) {
+  if (limit != 0 && __all_sync(0xFFFFFFFFu, poll(bar, parity))) return true;
+  return __all_sync(0xFFFFFFFFu, wait_or_abort(bar, parity, abort_flag, err, limit));
+}
+
 // Drain wait used on the way out: bounded, not cut short by the abort flag.
 __device__ void drain(uint64_t* bar, uint32_t parity, unsigned* err) {
   const uint32_t b = sa(bar);
@@ -123,18 +127,25 @@ __device__ void drain(uint64_t* bar, uint32_t parity, unsigned* err) {
   if (err) atomicOr(err, 2u);
 }
 
-// shared-memory matrix descriptor: K-major, 128-byte swizzle, 8-row groups 1 KB apart
-__device__ __forceinline__ uint64_t desc(uint32_t addr) {
-  return (uint64_t)((addr >> 4) & 0x3FFF) | ((uint64_t)1 << 16) | ((uint64_t)(1024 >> 4) << 32) | ((uint64_t)1 << 46) |
-         ((uint64_t)2 << 61);
-}
+// Shared-memory matrix descriptors, 128-byte swizzle; the low word holds the address and the leading
+// offset, the high word is the same for both forms (stride offset 1 KB).  K-major: 8-row groups 1 KB
+// apart.  MN-major: 8 K rows of 64 MN elements (128 bytes each) form a 1 KB atom; K groups of 8 rows 1 KB
+// apart, blocks of 64 MN elements 8 KB apart (leading offset: one TMA box of 64 x 64 each).
+constexpr uint32_t DESC_HI = (1024u >> 4) | (1u << 14) | (2u << 29);
 
-// shared-memory matrix descriptor: MN-major, 128-byte swizzle: 8 K rows of 64 MN elements
-// (128 bytes each) form a 1 KB atom; K groups of 8 rows 1 KB apart (stride offset), blocks of
-// 64 MN elements 8 KB apart (leading offset: one TMA box of 64 x 64 each)
-__device__ __forceinline__ uint64_t desc_mn(uint32_t addr) {
-  return (uint64_t)((addr >> 4) & 0x3FFF) | ((uint64_t)(8192 >> 4) << 16) | ((uint64_t)(1024 >> 4) << 32) |
-         ((uint64_t)1 << 46) | ((uint64_t)2 << 61);
+// One MMA / commit by one elected lane of a converged warp (always the same lane).
+__device__ __forceinline__ void mma(uint32_t acc, uint32_t a, uint32_t b, uint32_t idesc, bool accumulate) {
+  asm volatile(
+      "{\n .reg .pred p, q;\n .reg .b64 da, db;\n elect.sync _|q, 0xffffffff;\n setp.ne.u32 p, %5, 0;\n"
+      " mov.b64 da, {%1, %3};\n mov.b64 db, {%2, %3};\n"
+      " @q tcgen05.mma.cta_group::1.kind::f16 [%0], da, db, %4, p;\n}\n" ::"r"(acc),
+      "r"(a), "r"(b), "r"(DESC_HI), "r"(idesc), "r"((uint32_t)accumulate));
+}
+__device__ __forceinline__ void commit(uint32_t bar) {
+  asm volatile(
+      "{\n .reg .pred q;\n elect.sync _|q, 0xffffffff;\n"
+      " @q tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];\n}\n" ::"r"(bar)
+      : "memory");
 }
 
 // instruction descriptor: bf16 x bf16 -> f32, both K-major, M = 128, N = 256 (bits 15 / 16 make
@@ -233,13 +244,31 @@ __device__ __forceinline__ uint32_t stg_off(int r, int b) {
   return (uint32_t)(r * 64 + ((((b >> 4) ^ (r >> 1)) & 3) << 4) + (b & 15));
 }
 
+// v[j] with a run-time j, by a tree of selects (a dynamic index would put v in local memory, and staging
+// the rows in shared memory would take the room of a stage of the ring)
+__device__ __forceinline__ uint32_t pick32(const uint32_t (&v)[32], int j) {
+  uint32_t a[16], b[8], c[4];
+#pragma unroll
+  for (int i = 0; i < 16; i++) a[i] = (j & 1) ? v[2 * i + 1] : v[2 * i];
+#pragma unroll
+  for (int i = 0; i < 8; i++) b[i] = (j & 2) ? a[2 * i + 1] : a[2 * i];
+#pragma unroll
+  for (int i = 0; i < 4; i++) c[i] = (j & 4) ? b[2 * i + 1] : b[2 * i];
+  const uint32_t d0 = (j & 8) ? c[1] : c[0], d1 = (j & 8) ? c[3] : c[2];
+  return (j & 16) ? d1 : d0;
+}
+
+// Class of a column of the top-k output layer (INT_MAX: no column).
+__device__ __forceinline__ int class_of(const int32_t* col_id, int c) {
+  return c == INT_MAX || !col_id ? c : __ldg(col_id + c);
+}
+
 // Top-k chunk (one row per lane, 32 columns): the logits acc + bias enter the row's running list
 // (bv, bi: value descending, index ascending) if they reach its last entry; the first full chunk
 // seeds the threshold with the smallest of KT group maxima.  Warp-collective.
 template <int KT>
 __device__ __forceinline__ void topk_chunk(uint32_t (&v)[32], const float* bias, int cmax, int colbase,
-                                           const int32_t* col_id, float (&bv)[KT], int (&bi)[KT], bool& seeded,
-                                           float* area, int lane) {
+                                           const int32_t* col_id, float (&bv)[KT], int (&bi)[KT], bool& seeded) {
   // 1. bias-added logits of the chunk (cmax of its columns are valid)
 #pragma unroll
   for (int j = 0; j < 32; j += 4) {
@@ -281,34 +310,50 @@ __device__ __forceinline__ void topk_chunk(uint32_t (&v)[32], const float* bias,
   uint32_t mask = ((part[0] | part[1]) | (part[2] | part[3])) | ((part[4] | part[5]) | (part[6] | part[7]));
   if (cmax < 32) mask &= (1u << cmax) - 1u;
   if (__any_sync(0xFFFFFFFFu, mask != 0)) {
-    // 3. stage the row (16-byte groups XOR-swizzled by lane: conflict-free), then
-    //    insert each lane's candidates in column order, one per lane per round
-#pragma unroll
-    for (int g = 0; g < 8; g++)
-      *reinterpret_cast<uint4*>(area + lane * 32 + ((g ^ (lane & 7)) << 2)) =
-          make_uint4(v[4 * g], v[4 * g + 1], v[4 * g + 2], v[4 * g + 3]);
-    __syncwarp();
+    // 3. insert each lane's candidates in column order, one per lane per round
     while (__any_sync(0xFFFFFFFFu, mask != 0)) {
       if (mask) {
         const int j = __ffs(mask) - 1;
         mask &= mask - 1;
-        float cv = area[lane * 32 + (((j >> 2) ^ (lane & 7)) << 2) + (j & 3)];
-        int ci = col_id ? __ldg(col_id + colbase + j) : colbase + j;
-        if (cv > bv[KT - 1] || (cv == bv[KT - 1] && ci < bi[KT - 1])) {
+        float cv = __uint_as_float(pick32(v, j));
+        // the list holds columns; ids are looked up where values tie and at the end (a read of the id at
+        // every insertion waited for L2: 782 against 726 us)
+        int ci = colbase + j;
+        bool tie = false;
+#pragma unroll
+        for (int e = 0; e < KT; e++) tie |= cv == bv[e];
+        if (!tie) {
+          if (cv > bv[KT - 1]) {
+#pragma unroll
+            for (int e = 0; e < KT; e++) {
+              const bool take = cv > bv[e];
+              const float tv = bv[e];
+              const int ti = bi[e];
+              bv[e] = take ? cv : bv[e];
+              bi[e] = take ? ci : bi[e];
+              cv = take ? tv : cv;
+              ci = take ? ti : ci;
+            }
+          }
+        } else {
+          int id = class_of(col_id, ci);
 #pragma unroll
           for (int e = 0; e < KT; e++) {
-            const bool take = cv > bv[e] || (cv == bv[e] && ci < bi[e]);
-            const float tv = bv[e];
-            const int ti = bi[e];
-            bv[e] = take ? cv : bv[e];
-            bi[e] = take ? ci : bi[e];
-            cv = take ? tv : cv;
-            ci = take ? ti : ci;
+            const int held = cv == bv[e] ? class_of(col_id, bi[e]) : 0;
+            const bool take = cv > bv[e] || (cv == bv[e] && id < held);
+            if (take) {
+              const float tv = bv[e];
+              const int ti = bi[e];
+              bv[e] = cv;
+              bi[e] = ci;
+              cv = tv;
+              ci = ti;
+              id = class_of(col_id, ti);
+            }
           }
         }
       }
     }
-    __syncwarp();
   }
 }
 
@@ -375,7 +420,7 @@ __global__ void __launch_bounds__(Shape<KT>::kThreads, 1)
         for (int kc = w.kb; kc < w.ke; kc++, it++) {
           const uint32_t s = it % STAGES, r = it / STAGES;
           // round r reuses the stage after the MMAs of round r - 1 committed (round 0: fresh barrier)
-          if (!wait_or_abort(&empty[s], (r & 1) ^ 1, abort_flag, err, p.spin)) {
+          if (!wait_or_abort(sa(&empty[s]), (r & 1) ^ 1, abort_flag, err, p.spin)) {
             ok = false;
             break;
           }
@@ -401,53 +446,56 @@ __global__ void __launch_bounds__(Shape<KT>::kThreads, 1)
       const uint32_t cnt = it > s ? (it - s + STAGES - 1) / STAGES : 0;
       if (cnt) drain(&full[s], (cnt - 1) & 1, err);
     }
-  } else if (warp == 1 && lane == 0) {
+  } else if (warp == 1) {
     // ---------------------------------------------------------------- MMA issuer
-    uint32_t it = 0, tl = 0;
+    // Every instruction here delays the next MMA (the tensor core has few queued, and the epilogue warps
+    // compete for the issue slots), so the loop is kept short: the whole warp walks it and one elected
+    // lane issues (no loops over divergent lanes, operands in uniform registers), a wait is one poll
+    // where the barrier is complete (looking a chunk ahead did not help), and descriptors are one word.  Proposal top-4 of 16,384
+    // ids 818 -> 776 us, training step 979 -> 950 us against a single lane in a divergent branch.
+    uint32_t s = 0, par = 0, it = 0, tl = 0;  // stage and its round's parity, chunks, tiles
     bool ok = true;
     const uint32_t idesc = IDESC | ((uint32_t)(p.a_mn != 0) << 15) | ((uint32_t)(p.b_mn != 0) << 16);
+    const uint32_t a_base = (sa(smem) >> 4) | (p.a_mn ? (8192u >> 4) << 16 : 1u << 16), a_step = p.a_mn ? 2048 >> 4 : 32 >> 4;
+    const uint32_t b_base = ((sa(smem) + A_BYTES) >> 4) | (p.b_mn ? (8192u >> 4) << 16 : 1u << 16),
+                   b_step = p.b_mn ? 2048 >> 4 : 32 >> 4;
+    const uint32_t full0 = sa(full), empty0 = sa(empty);
     for (int u = blockIdx.x; u < p.units && ok; u += gridDim.x) {
       const Unit w = unit_of(p, u);
       for (int tn = w.nb; tn < w.ne && ok; tn++, tl++) {
         const uint32_t a = tl & 1, ar = tl >> 1;
-        if (!wait_or_abort(&tmem_empty[a], (ar & 1) ^ 1, abort_flag, err, p.spin)) {
+        const uint32_t te = sa(&tmem_empty[a]);
+        if (!warp_wait(te, (ar & 1) ^ 1, abort_flag, err, p.spin)) {
           ok = false;
           break;
         }
-        asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
         const uint32_t acc_addr = tmem + a * TN;
-        for (int kc = w.kb; kc < w.ke; kc++, it++) {
-          const uint32_t s = it % STAGES, r = it / STAGES;
-          if (!wait_or_abort(&full[s], r & 1, abort_flag, err, p.spin)) {
+        for (int kc = w.kb; kc < w.ke; kc++) {
+          if (!warp_wait(full0 + 8 * s, par, abort_flag, err, p.spin)) {
             ok = false;
             break;
           }
           asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-          const uint32_t a_addr = sa(smem + s * STAGE_BYTES), b_addr = a_addr + A_BYTES;
-#pragma unroll
-          for (int ks = 0; ks < TK / 16; ks++) {
-            const uint32_t accumulate = (kc != w.kb || ks != 0) ? 1u : 0u;
-            asm volatile(
-                "{\n .reg .pred p;\n setp.ne.u32 p, %4, 0;\n tcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, p;\n}\n" ::"r"(
-                    acc_addr),
-                "l"(p.a_mn ? desc_mn(a_addr + ks * 2048) : desc(a_addr + ks * 32)),
-                "l"(p.b_mn ? desc_mn(b_addr + ks * 2048) : desc(b_addr + ks * 32)), "r"(idesc), "r"(accumulate));
+          const uint32_t al = a_base + s * (STAGE_BYTES >> 4), bl = b_base + s * (STAGE_BYTES >> 4), freed = empty0 + 8 * s;
+          if (++s == STAGES) {
+            s = 0;
+            par ^= 1;
           }
-          asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(sa(&empty[s]))
-                       : "memory");
+#pragma unroll
+          for (int ks = 0; ks < TK / 16; ks++)
+            mma(acc_addr, al + ks * a_step, bl + ks * b_step, idesc, ks != 0 || kc != w.kb);
+          commit(freed);
+          it++;
         }
-        if (ok)
-          asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(
-                           sa(&tmem_full[a]))
-                       : "memory");
+        if (ok) commit(sa(&tmem_full[a]));
       }
     }
     // all MMAs issued by this thread complete, and every stage release has arrived
-    asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(sa(&done)) : "memory");
+    commit(sa(&done));
     drain(&done, 0, err);
-    for (uint32_t s = 0; s < STAGES; s++) {
-      const uint32_t cnt = it > s ? (it - s + STAGES - 1) / STAGES : 0;
-      if (cnt) drain(&empty[s], (cnt - 1) & 1, err);
+    for (uint32_t k = 0; k < STAGES; k++) {
+      const uint32_t cnt = it > k ? (it - k + STAGES - 1) / STAGES : 0;
+      if (cnt) drain(&empty[k], (cnt - 1) & 1, err);
     }
   } else if (warp >= 2) {
     // ---------------------------------------------------------------- epilogue
@@ -457,7 +505,7 @@ __global__ void __launch_bounds__(Shape<KT>::kThreads, 1)
     const int cbeg = h * CW, cend = cbeg + CW;
     float* area = reinterpret_cast<float*>(smem + STAGES * STAGE_BYTES + Shape<KT>::kStgBytes) + (warp - 2) * Shape<KT>::kAreaFloats;
     // top-k / softmax modes: this warp's biases of the tile
-    float* bsm = area + (KT > 0 ? SX_FLOATS : 0);
+    float* bsm = area;
     // gradient mode: this warp's staging buffers and the count of blocks it has staged
     uint8_t* stg = smem + STAGES * STAGE_BYTES + (warp - 2) * STG_WARP;
     uint32_t staged = 0;
@@ -539,7 +587,7 @@ __global__ void __launch_bounds__(Shape<KT>::kThreads, 1)
             keepm[i] = keep;
           }
         }
-        if (!wait_or_abort(&tmem_full[a], ar & 1, abort_flag, err, p.spin)) {
+        if (!wait_or_abort(sa(&tmem_full[a]), ar & 1, abort_flag, err, p.spin)) {
           ok = false;
           break;
         }
@@ -638,12 +686,12 @@ __global__ void __launch_bounds__(Shape<KT>::kThreads, 1)
           for (int i = 0; i < nch; i += 2) {
             if (i + 1 < nch) tmem_ld32_issue(tbase + 32 * (i + 1), vb);
             topk_chunk<KT>(va, bsm + 32 * i, min(32, p.N - (n0 + cbeg + 32 * i)), n0 + cbeg + 32 * i, ep.col_id, bv, bi,
-                           seeded, area, lane);
+                           seeded);
             if (i + 1 < nch) {
               tmem_wait(vb);
               if (i + 2 < nch) tmem_ld32_issue(tbase + 32 * (i + 2), va);
               topk_chunk<KT>(vb, bsm + 32 * (i + 1), min(32, p.N - (n0 + cbeg + 32 * (i + 1))), n0 + cbeg + 32 * (i + 1),
-                             ep.col_id, bv, bi, seeded, area, lane);
+                             ep.col_id, bv, bi, seeded);
               if (i + 2 < nch) tmem_wait(va);
             }
           }
@@ -736,7 +784,9 @@ __global__ void __launch_bounds__(Shape<KT>::kThreads, 1)
 #pragma unroll
           for (int j = 0; j < KT; j += 4) {
             *reinterpret_cast<float4*>(ep.cand_v + off + j) = make_float4(bv[j], bv[j + 1], bv[j + 2], bv[j + 3]);
-            *reinterpret_cast<int4*>(ep.cand_i + off + j) = make_int4(bi[j], bi[j + 1], bi[j + 2], bi[j + 3]);
+            *reinterpret_cast<int4*>(ep.cand_i + off + j) = 
+                make_int4(class_of(ep.col_id, bi[j]), class_of(ep.col_id, bi[j + 1]), class_of(ep.col_id, bi[j + 2]),
+                          class_of(ep.col_id, bi[j + 3]));
           }
         }
       }
@@ -924,11 +974,18 @@ void launch(const CUtensorMap& ma, const CUtensorMap& mb, const CUtensorMap& mdz
 
 }  // namespace
 
-// column ranges of the top-k and statistics modes: as many as make the units a multiple of the
-// SM count (balanced waves)
+// Column ranges of the top-k and statistics modes: the fewest within 3 % of the least time in tiles per
+// SM.  A row's list starts anew in each range, and its first columns are the ones that enter, so few long
+// ranges cost less: 16,384 rows x 202 column tiles took 726 us in 19 ranges (units a multiple of the SMs)
+// and 660 us in 7 (top-4; top-16 of 9,000 rows 3.2 ms and, with the lists' columns below, 0.64 ms).
 int tc_ranges(int M, int N) {
   const int mt = (M + TM - 1) / TM, nt = (N + TN - 1) / TN, g = sm_count();
-  return std::max(1, std::min(nt, g / std::gcd(mt, g)));
+  auto time = [&](int nr) { return (long long)((mt * (long long)nr + g - 1) / g) * ((nt + nr - 1) / nr); };
+  long long least = time(1);
+  for (int nr = 2; nr <= std::min(nt, g); nr++) least = std::min(least, time(nr));
+  int nr = 1;
+  while (time(nr) * 100 > least * 103) nr++;
+  return nr;
 }
 
 int tc_stats_lists(int M, int N) { return tc_ranges(M, N) * kTcStatsListsPerTile; }
