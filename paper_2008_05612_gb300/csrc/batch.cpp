@@ -211,7 +211,7 @@ extern "C" int hp_batch_plan_create(const hp_structs* const* libs, const uint64_
   // plans (tables are uploaded here, before capture begins) and their device blocks
   std::vector<hp::PhenParams*> prms;
   std::vector<int> shape_r, shape_t;
-  for (const int c : {14, 13, 12, 11}) {
+  for (const int c : {14, 12, 11}) {
     if (rc != HP_OK) break;
     std::vector<const hp_structs*> l;
     std::vector<uint64_t> bg, ct;

@@ -144,8 +144,14 @@ struct Cfg {
   // words per record: a multiple of 4 that is odd in 16-byte units (conflict-free 16-byte stores)
   static constexpr int CSTRIDE = ((CS_RAW / 4) % 2 == 1) ? CS_RAW : CS_RAW + 4;
   // pass 2 reads word j of 32 consecutive records (one per lane): an odd stride in words keeps
-  // those loads conflict-free, and the records are written with 4-byte stores
-  static constexpr int CS2 = CS_RAW | 1;
+  // those loads conflict-free, and the records are written with 4-byte stores.  Where the shared
+  // memory has room (tiles of up to 128) its records hold the P tree sums instead of the R - 1 tree
+  // coefficients: a candidate's score is then three reads and two adds instead of 2 + R - 1 reads and R + 1
+  // adds and selects (5x5, where two thirds of
+  // the sequences get here: 2.42 -> 2.14 ms).
+  static constexpr bool kTreeSums = T_ <= 128;
+  static constexpr int CS2_RAW = TP_OFF + (kTreeSums ? P : TP_WORDS);
+  static constexpr int CS2 = CS2_RAW | 1;
   static constexpr int kCoefWords = 2 * T * (CSTRIDE > CS2 ? CSTRIDE : CS2);
   static constexpr int kStateWords = 2 * P * THREADS;
   static_assert(T <= THREADS, "one producer thread per conformation of a tile");
@@ -215,8 +221,18 @@ __device__ __forceinline__ void produce_work(const hp::PhenInst& in, unsigned* e
         if (P2) {
 #pragma unroll
           for (int w = 0; w < K::NW; w++) c[K::WT_OFF + w] = wt[w] * 0x10001u;
+          if (K::kTreeSums) {
+            uint32_t sums[K::P];
+            sums[0] = 0;
 #pragma unroll
-          for (int j = 0; j < R - 1; j++) c[K::TP_OFF + j] = tp[j];
+            for (int v = 0; v < K::P; v++) {
+              if (v) sums[v] = sums[v ^ (1 << (31 - __clz(v)))] + tp[31 - __clz(v)];
+              c[K::TP_OFF + v] = sums[v];
+            }
+          } else {
+#pragma unroll
+            for (int j = 0; j < R - 1; j++) c[K::TP_OFF + j] = tp[j];
+          }
         } else {
 #pragma unroll
           for (int w = 0; w < K::NW; w += 4)
@@ -230,7 +246,7 @@ __device__ __forceinline__ void produce_work(const hp::PhenInst& in, unsigned* e
         // padding conformation: every score 0, below every real (biased) score
         if (P2) {
 #pragma unroll
-          for (int k = 0; k < K::CS_RAW; k++) c[k] = 0u;
+          for (int k = 0; k < K::CS2_RAW; k++) c[k] = 0u;
         } else {
 #pragma unroll
           for (int k = 0; k < K::CS_RAW; k += 4) *reinterpret_cast<uint4*>(c + k) = make_uint4(0, 0, 0, 0);
@@ -566,8 +582,12 @@ __global__ void __launch_bounds__(K::THREADS, 1) phenotype_kernel(const __grid_c
         for (int sc = 0; sc < T; sc++) {
           const uint32_t* cs = cbuf + sc * K::CS2;
           uint32_t x = cs[src] + cs[K::WT_OFF + wo];
+          if (K::kTreeSums) {
+            x += cs[K::TP_OFF + v];
+          } else {
 #pragma unroll
-          for (int j = 0; j < R - 1; j++) x += ((v >> j) & 1) ? cs[K::TP_OFF + j] : 0u;
+            for (int j = 0; j < R - 1; j++) x += ((v >> j) & 1) ? cs[K::TP_OFF + j] : 0u;
+          }
           const uint32_t xf = (x >> (16 * h)) & 0xFFFFu;
           if (xf == want) {  // padding scores 0 never match
             first = min(first, sc);
@@ -592,9 +612,13 @@ __global__ void __launch_bounds__(K::THREADS, 1) phenotype_kernel(const __grid_c
         for (int i = 0; i < T; i += 32) {
           const uint32_t* cs = cbuf + (i + lane) * K::CS2;
           uint32_t x = cs[src] + cs[K::WT_OFF + wo];
+          if (K::kTreeSums) {
+            x += cs[K::TP_OFF + v];
+          } else {
 #pragma unroll
-          for (int j = 0; j < R - 1; j++)
-            if ((v >> j) & 1) x += cs[K::TP_OFF + j];
+            for (int j = 0; j < R - 1; j++)
+              if ((v >> j) & 1) x += cs[K::TP_OFF + j];
+          }
           const uint32_t xf = (x >> (16 * h)) & 0xFFFFu;
           const uint32_t bal = __ballot_sync(0xFFFFFFFFu, xf == want);  // padding scores 0 never match
           if (bal) first = min(first, i + __ffs(bal) - 1);
@@ -783,9 +807,12 @@ int shape_grid_or_launch(const hp::PhenParams& prm, cudaStream_t stream, unsigne
 
 namespace hp {
 
+// 13 free even residues take the 12-role shape too (two items per odd pattern): a 13-role shape (8 warps,
+// 128 conformations per tile) took 124.1 ms for 2^25 ids of 3x3x3 where this one takes 119.1, 70.5 against 68.2
+// for 2^25 ids of 6x6, and 2.14 against 2.12 for 5x5.
 void small_roles_shape(int max_ne_free, int* roles, int* reg_bits, int* tile) {
-  *roles = max_ne_free >= kRoles ? kRoles : std::max(max_ne_free, 11);
-  if (*roles == 13 || *roles == 12) {
+  *roles = max_ne_free >= kRoles ? kRoles : max_ne_free >= 12 ? 12 : 11;
+  if (*roles == 12) {
     *reg_bits = 5;
     *tile = 128;
   } else if (*roles == 11) {
@@ -815,7 +842,6 @@ int grid_or_launch(const PhenParams& prm, int reg_bits, int tile, cudaStream_t s
   if (prm.gap2 > 2u) return shape_grid_or_launch<Cfg<5, 256>, true>(prm, stream, grid_limit, grid, launch);
   // fewer roles per CTA: one compiled shape each (small_roles_shape)
   switch (prm.roles) {
-    case 13: return shape_grid_or_launch<Cfg<5, 128, 13>>(prm, stream, grid_limit, grid, launch);
     case 12: return shape_grid_or_launch<Cfg<5, 128, 12>>(prm, stream, grid_limit, grid, launch);
     case 11: return shape_grid_or_launch<Cfg<4, 64, 11>>(prm, stream, grid_limit, grid, launch);
     case kRoles: break;
@@ -899,7 +925,7 @@ int half_tables(const hp_structs* cs, DevTables** out) {
 
 int plan_phenotype(const hp_structs* const* libs, const uint64_t* begins, const uint64_t* counts, int n,
                    int32_t* const* d_phen, int32_t* const* d_aux, int tile, PhenParams& prm, int roles) {
-  if (roles != kRoles && roles != 13 && roles != 12 && roles != 11) return fail(HP_EINVAL, "unsupported role count");
+  if (roles != kRoles && roles != 12 && roles != 11) return fail(HP_EINVAL, "unsupported role count");
   prm.roles = roles;
   if (n < 1 || n > kPhenMaxInst)
     return fail(HP_EINVAL, "a batch holds 1 to " + std::to_string(kPhenMaxInst) + " instances");
@@ -1014,7 +1040,7 @@ int run_phenotype(const hp_structs* const* libs, const uint64_t* begins, const u
     int rc = role_classes(libs, begins, counts, n, d_phen, tile, cls);
     if (rc != HP_OK) return rc;
     if (std::any_of(cls.begin(), cls.end(), [&](int c) { return c != cls[0]; })) {
-      for (const int c : {kRoles, 13, 12, 11}) {
+      for (const int c : {kRoles, 12, 11}) {
         std::vector<const hp_structs*> l;
         std::vector<uint64_t> b, k;
         std::vector<int32_t*> o, a;
@@ -1091,8 +1117,9 @@ namespace {
 // odd one, which pays where an aligned block leaves many even residues free: a block of 2^m ids has
 // ceil(m / 2), and a CTA always evaluates 2^roles patterns.  The aligned blocks of a range grow and
 // then shrink, so the blocks of at least 2^m ids are one run; the m with the least estimated time is
-// taken.  Rates measured on 3x3x3, 2x3x4, 6x6 (scores/s): map kernel 3.5e13 with 14 roles, 3.2e13 and 3.0e13
-// with 13 and 12, 1.55e13 with 11; scan 1 / (7.9e-14 s max(1, pairs / 150) conformations + 0.62 ns) per id.
+// taken.  Rates measured on 3x3x3, 2x3x4, 6x6 (scores/s): map kernel 3.5e13 with 14 roles, 2.9e13 with 12,
+// 2.15e13 with 11; scan 7.9e-14 s max(1, pairs / 150) conformations + 0.62 ns per id.  2^20 ids of 3x3x3 take 10.4 ms
+// by the map kernel and 9.0 by the scan, 2^21 10.6 and 18.
 void split_range(const hp_structs* s, uint64_t begin, uint64_t count, int gap_threshold, uint64_t* map_begin,
                  uint64_t* map_end) {
   constexpr double kSms = 152;
@@ -1110,7 +1137,7 @@ void split_range(const hp_structs* s, uint64_t begin, uint64_t count, int gap_th
   }
   const double pairs = (double)s->NE * s->NO - (s->N - 1);  // pairs that may be in contact
   const double scan_id = 0.62e-9 + 7.9e-14 * std::max(1.0, pairs / 150.0) * s->S_dir;
-  double best = 25e-6 + count * scan_id;  // no block to the map kernel
+  double best = 40e-6 + count * scan_id;  // no block to the map kernel
   *map_begin = *map_end = begin;
   for (int mmin = 0; mmin < 63; mmin++) {
     uint64_t lo = end, hi = end, ids = 0;
@@ -1132,12 +1159,12 @@ void split_range(const hp_structs* s, uint64_t begin, uint64_t count, int gap_th
         const int ne = std::min((b.m + 1) / 2, s->NE);
         items += std::ldexp(half ? 0.51 : 1.0, b.m - std::min(ne, roles));
       }
-    const double ctas = roles == 14 ? 1 : roles == 13 ? 2 : roles == 12 ? 2 : 4;
-    const double rate = roles == 14 ? 3.5e13 : roles == 13 ? 3.2e13 : roles == 12 ? 3.0e13 : 1.55e13;
+    const double ctas = roles == 14 ? 1 : roles == 12 ? 2 : 4;
+    const double rate = roles == 14 ? 3.5e13 : roles == 12 ? 2.9e13 : 2.15e13;
     const double item = std::ldexp((double)s->S_dir, roles) * kSms * ctas / rate + 20e-6;
     const double waves = std::max(1.0, items / (kSms * ctas));
     const uint64_t rest = count - ids;
-    const double cost = 25e-6 + waves * item + (rest ? 25e-6 + rest * scan_id : 0.0);
+    const double cost = 25e-6 + waves * item + (rest ? 40e-6 + rest * scan_id : 0.0);
     if (cost < best) {
       best = cost;
       *map_begin = lo;

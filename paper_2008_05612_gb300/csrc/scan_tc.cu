@@ -436,6 +436,12 @@ __global__ void __launch_bounds__(256) scan_tc_resolve(const ResolveParams p) {
     join(b, s, __shfl_xor_sync(0xFFFFFFFFu, grp, d));
   }
   good = __all_sync(0xFFFFFFFFu, good);
+  // another group within T of the best and no label wanted: not a fold, whatever the group holds (95 % of
+  // 3x3x3's ids); scores are whole numbers
+  if (good && !p.aux && !p.gap && sec + 10.f * p.C >= 0.f && best - sec < (float)p.T) {
+    if (lane == 0) p.phen[row] = -1;
+    return;
+  }
   int M = 0, second = -1, first = 0;  // best score, second best (< 0: none), lowest minimiser
   if (good) {
     const int c = kGroup * grp + lane;
