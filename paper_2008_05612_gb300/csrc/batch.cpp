@@ -225,7 +225,9 @@ extern "C" int hp_batch_plan_create(const hp_structs* const* libs, const uint64_
       }
     if (l.empty()) continue;
     int r2 = r, t2 = t, roles = 14;
-    if (c != 14) hp::small_roles_shape(c, &roles, &r2, &t2);
+    int min_conf = l[0]->S_dir;
+    for (const hp_structs* b : l) min_conf = std::min(min_conf, (int)b->S_dir);
+    if (c != 14) hp::small_roles_shape(c, min_conf, &roles, &r2, &t2);
     hp::PhenParams* prm = new (std::nothrow) hp::PhenParams();
     if (!prm) {
       rc = hp::fail(HP_ENOMEM, "hp_batch_plan_create: out of host memory");

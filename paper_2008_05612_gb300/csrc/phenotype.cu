@@ -568,9 +568,12 @@ __global__ void __launch_bounds__(K::THREADS, 1) phenotype_kernel(const __grid_c
       const uint32_t* cbuf = coefbuf + b * T * K::CS2;
       const int e0 = woff[t], e1 = woff[t + 1];
       // a tile with at least 32 candidates per warp: each lane scores one candidate against every
-      // conformation of the tile (no votes, independent steps); the rest one candidate per warp
-      const int nlane = (e1 - e0) / (32 * K::NW) * (32 * K::NW);
+      // conformation of the tile (no votes, independent steps); the rest one candidate per warp, or
+      // where it is more than 16 a warp in lanes too (a round of lanes costs as much as 15 of them)
+      const int rest = (e1 - e0) % (32 * K::NW);
+      const int nlane = e1 - e0 - (K::kTreeSums && rest > 16 * K::NW ? 0 : rest);
       for (int base = e0 + 32 * warp; base < e0 + nlane; base += 32 * K::NW) {
+        if (base + lane >= e0 + nlane) continue;
         const uint32_t ent = wl[base + lane];
         const int owner = (int)(ent >> 6), c = (int)(ent & 63u), v = c >> 1, h = c & 1;
         const int src = owner & 31, wo = owner >> 5;
@@ -578,7 +581,7 @@ __global__ void __launch_bounds__(K::THREADS, 1) phenotype_kernel(const __grid_c
         const uint32_t sfld = best16[fi];
         const uint32_t want = sfld & 0xFFFEu;
         int count = 0, first = 0x7FFFFFFF;
-#pragma unroll 4
+#pragma unroll (K::kTreeSums ? 16 : 4)  // (4 in the small shapes: 5x5 2.12 ms, 16: 1.96; few warps hide the reads)
         for (int sc = 0; sc < T; sc++) {
           const uint32_t* cs = cbuf + sc * K::CS2;
           uint32_t x = cs[src] + cs[K::WT_OFF + wo];
@@ -810,14 +813,17 @@ namespace hp {
 // 13 free even residues take the 12-role shape too (two items per odd pattern): a 13-role shape (8 warps,
 // 128 conformations per tile) took 124.1 ms for 2^25 ids of 3x3x3 where this one takes 119.1, 70.5 against 68.2
 // for 2^25 ids of 6x6, and 2.14 against 2.12 for 5x5.
-void small_roles_shape(int max_ne_free, int* roles, int* reg_bits, int* tile) {
+// The 11-role shape takes tiles of 128 conformations instead of 64 for libraries of 2^16 or more, where fewer
+// merges per conformation count more than cheaper pass-2 candidates: 2^21 ids of 3x3x3 (103,346
+// conformations) 10.57 -> 8.93 ms, but 2^22 of 6x6 (57,337) 11.46 -> 11.88 and 4x5 (503) 0.19 -> 0.23.
+void small_roles_shape(int max_ne_free, int min_conf, int* roles, int* reg_bits, int* tile) {
   *roles = max_ne_free >= kRoles ? kRoles : max_ne_free >= 12 ? 12 : 11;
   if (*roles == 12) {
     *reg_bits = 5;
     *tile = 128;
   } else if (*roles == 11) {
     *reg_bits = 4;
-    *tile = 64;
+    *tile = min_conf >= (1 << 16) ? 128 : 64;
   }
 }
 
@@ -840,10 +846,12 @@ int grid_or_launch(const PhenParams& prm, int reg_bits, int tile, cudaStream_t s
                    unsigned* grid, bool launch) {
   // thresholds above 1 have one compiled shape (the default)
   if (prm.gap2 > 2u) return shape_grid_or_launch<Cfg<5, 256>, true>(prm, stream, grid_limit, grid, launch);
-  // fewer roles per CTA: one compiled shape each (small_roles_shape)
+  // fewer roles per CTA (small_roles_shape)
   switch (prm.roles) {
     case 12: return shape_grid_or_launch<Cfg<5, 128, 12>>(prm, stream, grid_limit, grid, launch);
-    case 11: return shape_grid_or_launch<Cfg<4, 64, 11>>(prm, stream, grid_limit, grid, launch);
+    case 11:
+      return tile == 128 ? shape_grid_or_launch<Cfg<4, 128, 11>>(prm, stream, grid_limit, grid, launch)
+                         : shape_grid_or_launch<Cfg<4, 64, 11>>(prm, stream, grid_limit, grid, launch);
     case kRoles: break;
     default: return fail(HP_EINVAL, "unsupported role count");
   }
@@ -1017,7 +1025,7 @@ int role_classes(const hp_structs* const* libs, const uint64_t* begins, const ui
     }
     int max_ne = 0, r = 0, t = 0;
     for (int k = 0; k < tmp->nblocks; k++) max_ne = std::max(max_ne, (int)tmp->blocks[k].ne_free);
-    small_roles_shape(max_ne, &cls[i], &r, &t);
+    small_roles_shape(max_ne, libs[i]->S_dir, &cls[i], &r, &t);
   }
   delete tmp;
   return HP_OK;
@@ -1069,7 +1077,9 @@ int run_phenotype(const hp_structs* const* libs, const uint64_t* begins, const u
     int max_ne = 0;
     for (int i = 0; i < prm->nblocks; i++) max_ne = std::max(max_ne, (int)prm->blocks[i].ne_free);
     int roles = kRoles;
-    small_roles_shape(max_ne, &roles, &reg_bits, &tile);
+    int min_conf = libs[0]->S_dir;
+    for (int i = 1; i < n; i++) min_conf = std::min(min_conf, (int)libs[i]->S_dir);
+    small_roles_shape(max_ne, min_conf, &roles, &reg_bits, &tile);
     if (roles != kRoles) rc = plan_phenotype(libs, begins, counts, n, d_phen, d_aux, tile, *prm, roles);
   }
   prm->gap2 = 2u * (uint32_t)gap_threshold;
@@ -1118,8 +1128,8 @@ namespace {
 // ceil(m / 2), and a CTA always evaluates 2^roles patterns.  The aligned blocks of a range grow and
 // then shrink, so the blocks of at least 2^m ids are one run; the m with the least estimated time is
 // taken.  Rates measured on 3x3x3, 2x3x4, 6x6 (scores/s): map kernel 3.5e13 with 14 roles, 2.9e13 with 12,
-// 2.15e13 with 11; scan 7.9e-14 s max(1, pairs / 150) conformations + 0.62 ns per id.  2^20 ids of 3x3x3 take 10.4 ms
-// by the map kernel and 9.0 by the scan, 2^21 10.6 and 18.
+// 2.15e13 with 11 (2.5e13 with tiles of 128); scan 7.9e-14 s max(1, pairs / 150) conformations + 0.62 ns per id.  2^20 ids of 3x3x3 take 9.0 ms by
+// the scan, and 2^21 8.9 by the map kernel and 18 by the scan.
 void split_range(const hp_structs* s, uint64_t begin, uint64_t count, int gap_threshold, uint64_t* map_begin,
                  uint64_t* map_end) {
   constexpr double kSms = 152;
@@ -1151,7 +1161,7 @@ void split_range(const hp_structs* s, uint64_t begin, uint64_t count, int gap_th
       }
     if (!ids) break;
     int roles = kRoles, r = 0, t = 0;
-    if (gap_threshold == 1) small_roles_shape(max_ne, &roles, &r, &t);
+    if (gap_threshold == 1) small_roles_shape(max_ne, s->S_dir, &roles, &r, &t);
     double items = 0;
     for (const Block& b : blocks)
       if (b.m >= mmin) {
@@ -1160,7 +1170,7 @@ void split_range(const hp_structs* s, uint64_t begin, uint64_t count, int gap_th
         items += std::ldexp(half ? 0.51 : 1.0, b.m - std::min(ne, roles));
       }
     const double ctas = roles == 14 ? 1 : roles == 12 ? 2 : 4;
-    const double rate = roles == 14 ? 3.5e13 : roles == 12 ? 2.9e13 : 2.15e13;
+    const double rate = roles == 14 ? 3.5e13 : roles == 12 ? 2.9e13 : t == 128 ? 2.5e13 : 2.15e13;
     const double item = std::ldexp((double)s->S_dir, roles) * kSms * ctas / rate + 20e-6;
     const double waves = std::max(1.0, items / (kSms * ctas));
     const uint64_t rest = count - ids;
