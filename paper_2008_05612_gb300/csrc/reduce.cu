@@ -171,7 +171,7 @@ __device__ __forceinline__ unsigned tile_root(const uint16_t* par, unsigned x) {
 
 // ---------------------------------------------------------------- passes over the flips
 
-// Eq. 2 numerators in passes over the map, each reading it once.  A block is 2^kRobTileBits ids
+// Eq. 2 numerators in passes over the map, each reading it once.  A block is 2^13 ids (kRobTileBits)
 // in shared memory: 2^c consecutive ids times every combination of the pass's h bits
 // (c + h = kRobTileBits), the other bits of the id fixed by the block index.  The first pass
 // takes 2^13 consecutive ids and counts the flips of bits 0..12; each later pass counts the flips
@@ -227,6 +227,11 @@ __device__ __forceinline__ void phi_add(const hp::PhiTable& t, uint32_t key, uns
 // all flips through global labels took 67 + 566 + 178 us.
 enum FlipWork { kRobustness, kPhi, kJoinFirst, kJoin };
 
+// log2 of the ids per block (at most).  The phi table's inserts wait for L2, so its passes take half-size
+// blocks and more CTAs per SM: 2^25 ids 522 -> 410 us; the other passes are as fast or faster (Eq. 2 228 against
+// 247 us) with the longer runs of contiguous ids.
+__host__ __device__ constexpr int block_bits(int work) { return work == kPhi ? kRobTileBits - 1 : kRobTileBits; }
+
 template <int WORK>
 __global__ void __launch_bounds__(kRobThreads) flip_pass(const int32_t* __restrict__ phen, int S, const RobPass P,
                                                                unsigned long long nblocks, int replicas,
@@ -238,7 +243,7 @@ __global__ void __launch_bounds__(kRobThreads) flip_pass(const int32_t* __restri
   extern __shared__ int32_t tiles[];  // two blocks, then the list of a block's genotypes that fold
   __shared__ unsigned long long hoff[1 << kRobMaxPassBits];
   __shared__ unsigned nlist;
-  constexpr int kIds = 1 << kRobTileBits;
+  constexpr int kIds = 1 << block_bits(WORK);
   uint16_t* list = reinterpret_cast<uint16_t*>(tiles + 2 * kIds);
   static_assert(kRobTileBits <= 16, "list entries are 16-bit local indices");
   for (int i = threadIdx.x; i < (1 << P.h); i += blockDim.x) {
@@ -581,16 +586,24 @@ extern "C" int hp_robustness(const int32_t* d_phen, int32_t N, int32_t S, uint64
 
 namespace hp {
 
-// Ids per block: 2^13, or fewer for small maps, so that they still have 2^7 blocks or so to spread over
+// CTAs of a pass: as many as are resident (they walk the blocks), at most one per block.
+template <class Kernel>
+unsigned pass_grid(Kernel kernel, size_t smem, unsigned long long blocks) {
+  int per_sm = 0;
+  if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kernel, kRobThreads, smem) != cudaSuccess || per_sm < 1) per_sm = 1;
+  return (unsigned)std::min<unsigned long long>(blocks, (unsigned long long)sm_count() * per_sm);
+}
+
+// log2 of the ids per block: `most`, or less for small maps, so that they still have 2^7 blocks or so to spread over
 // the SMs and one later pass (4x4, 2^16 ids: Eq. 2 passes 20 -> 12 us,
 // networks 41 + 25 -> 10 + 18 us, against blocks of 2^13).
-int flip_block_bits(int N) { return std::min(N, std::max(9, std::min(kRobTileBits, N - 8))); }
+int flip_block_bits(int N, int most) { return std::min(N, std::max(9, std::min(most, N - 8))); }
 
 // The passes over the flips of an N-bit map: bits [0, k) first, then the high bits [k, N) in
 // near-equal groups of at most kRobMaxPassBits, each with the k - h lowest bits
 // contiguous.
-std::vector<RobPass> flip_passes(int N) {
-  const int k = flip_block_bits(N);
+std::vector<RobPass> flip_passes(int N, int most) {
+  const int k = flip_block_bits(N, most);
   std::vector<RobPass> plan;
   {
     RobPass p{};
@@ -618,16 +631,17 @@ std::vector<RobPass> flip_passes(int N) {
 cudaError_t launch_robustness(const int32_t* d_phen, int N, int S, unsigned long long* neutral,
                               unsigned long long* to_del, unsigned long long* negcount, unsigned* err, cudaStream_t st,
                               const PhiTable* phi) {
-  const unsigned long long blocks = 1ull << (N - flip_block_bits(N));
-  const size_t smem = 2 * (sizeof(int32_t) << kRobTileBits) + (sizeof(uint16_t) << kRobTileBits);
+  const int most = block_bits(phi ? kPhi : kRobustness);
+  const unsigned long long blocks = 1ull << (N - flip_block_bits(N, most));
+  const size_t smem = 2 * (sizeof(int32_t) << most) + (sizeof(uint16_t) << most);
   const auto pass = phi ? flip_pass<kPhi> : flip_pass<kRobustness>;
   const PhiTable table = phi ? *phi : PhiTable{};
   cudaError_t e = cudaFuncSetAttribute(pass, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
   if (e != cudaSuccess) return e;
-  const std::vector<RobPass> plan = flip_passes(N);
+  const std::vector<RobPass> plan = flip_passes(N, most);
   // a few CTAs per SM walking the blocks (shared memory: two blocks each), counting into
   // replicated counters (stream-ordered scratch; without it, straight into neutral / to_del)
-  const unsigned grid = (unsigned)std::min<unsigned long long>(blocks, (unsigned long long)sm_count() * 2);
+  const unsigned grid = pass_grid(pass, smem, blocks);
   unsigned long long* rep = nullptr;
   const size_t rep_bytes = sizeof(unsigned long long) * (2 * kRobReplicas * (size_t)S + 2);
   if (cudaMallocAsync(&rep, rep_bytes, st) != cudaSuccess || cudaMemsetAsync(rep, 0, rep_bytes, st) != cudaSuccess) {
@@ -665,19 +679,18 @@ extern "C" int hp_neutral_components(const int32_t* d_phen, int32_t N, int32_t S
   if (e != cudaSuccess) return hp::cuda_fail(e, "hp_neutral_components: cudaMallocAsync");
   cudaMemsetAsync(err, 0, sizeof(unsigned), st);
   cudaMemsetAsync(d_ncomp, 0, sizeof(uint64_t) * (size_t)S, st);
-  const unsigned long long total = 1ull << N, blocks = total >> hp::flip_block_bits(N);
-  const unsigned pgrid = (unsigned)std::min<unsigned long long>(blocks, (unsigned long long)sm_count() * 2);
+  const unsigned long long total = 1ull << N, blocks = total >> hp::flip_block_bits(N, kRobTileBits);
   const size_t smem = 2 * (sizeof(int32_t) << kRobTileBits) + (sizeof(uint16_t) << kRobTileBits);
   const size_t smem1 = smem + (sizeof(uint16_t) << kRobTileBits);  // and the block's parents
   e = cudaFuncSetAttribute(flip_pass<kJoinFirst>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem1);
   if (e == cudaSuccess) e = cudaFuncSetAttribute(flip_pass<kJoin>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
   if (e == cudaSuccess) {
-    for (const RobPass& p : hp::flip_passes(N)) {
+    for (const RobPass& p : hp::flip_passes(N, kRobTileBits)) {
       if (p.first)
-        flip_pass<kJoinFirst><<<pgrid, kRobThreads, smem1, st>>>(d_phen, S, p, blocks, 1, nullptr, nullptr, nullptr, err,
+        flip_pass<kJoinFirst><<<hp::pass_grid(flip_pass<kJoinFirst>, smem1, blocks), kRobThreads, smem1, st>>>(d_phen, S, p, blocks, 1, nullptr, nullptr, nullptr, err,
                                                                   hp::PhiTable{}, d_label);
       else
-        flip_pass<kJoin><<<pgrid, kRobThreads, smem, st>>>(d_phen, S, p, blocks, 1, nullptr, nullptr, nullptr, err,
+        flip_pass<kJoin><<<hp::pass_grid(flip_pass<kJoin>, smem, blocks), kRobThreads, smem, st>>>(d_phen, S, p, blocks, 1, nullptr, nullptr, nullptr, err,
                                                             hp::PhiTable{}, d_label);
     }
     const unsigned grid = (unsigned)std::min<unsigned long long>((total + 1023) / 1024, (unsigned long long)sm_count() * 16);
