@@ -91,13 +91,18 @@ void hp_structs_free(hp_structs* s);
  *                  [2, 2^20] run a variant of the map kernel that also keeps
  *                  the second-best tile maximum, always in the default shape
  *                  (reg_bits 5, tile 256); < 1 or > 2^20 give HP_EINVAL.
+ *                  Without a shape set on the library (hp_set_tile_cfg), the
+ *                  blocks of the range that are too short for the map kernel
+ *                  (or the whole range) are scored on the tensor cores; the
+ *                  results are the same.
  *   d_phen:        device int32[seq_count]; d_phen[k] = phenotype of
  *                  seq_begin + k: class id, or -1.
  *   d_argmin_aux:  optional device int32[seq_count] (NULL to skip): class of
  *                  the lowest-index conformation reaching the minimum energy,
  *                  tied or not (training labels for the learned proposal).
- * seq_begin + seq_count must not exceed 2^N.  Allocates a small stream-
- * ordered scratch block (work counter and error word) per call and
+ * seq_begin + seq_count must not exceed 2^N.  Allocates stream-ordered
+ * scratch per call (control words and work lists of the map kernel, at most
+ * 27 MB of partial results of the tensor-core scan) and
  * synchronises `stream` (it reads the error word back: HP_ETIMEOUT when a
  * bounded device wait gave up, see hp_set_wait_limit). */
 int hp_phenotype_map(const hp_structs* s, uint64_t seq_begin, uint64_t seq_count, int32_t gap_threshold,
@@ -164,9 +169,12 @@ int hp_batch_plan_status(hp_batch_plan* plan, void* stream);
 void hp_batch_plan_free(hp_batch_plan* plan);
 
 /* Ground state of an arbitrary list of sequence ids (e.g. a seeded sample,
- * the paper's sampling mode of Table 3), one warp per sequence, with optional
- * exact bound pruning seeded by candidate conformations (the learned
- * proposal).  With A_s(h) = sum_i h_i c_i(s) and B the HH-contact count,
+ * the paper's sampling mode of Table 3).  Every conformation is scored on the
+ * tensor cores (stream-ordered scratch of at most 27 MB; a capture records
+ * it), except in small scans (at most 1,024 conformations and n times these at
+ * most 2^22), where its table or scratch does not fit, and in calls with both
+ * d_cand and d_counters: these run one warp per sequence, with optional exact
+ * bound pruning seeded by candidate conformations (the learned proposal).  With A_s(h) = sum_i h_i c_i(s) and B the HH-contact count,
  * -E = 10 A + 3 B <= 10 A + 3 min(C, floor(A/2)) (Eq. 1, Table 1 x 10); A
  * depends on a conformation only through its contact-count vector, so the
  * bound is taken once per group of conformations sharing that vector, and a
@@ -178,7 +186,8 @@ void hp_batch_plan_free(hp_batch_plan* plan);
  *   d_phen:     device int32[n] phenotypes; d_aux: device int32[n] class of
  *               the lowest-index minimum (or NULL);
  *   d_counters: device uint64[2] (or NULL): conformations evaluated exactly
- *               and group bounds evaluated are ADDED to [0] and [1].
+ *               and group bounds evaluated are ADDED to [0] and [1] (n times
+ *               the conformations and 0 without candidates).
  * Stream-ordered; does not synchronise.  No counterpart in the paper beyond
  * its sampled kernel (Appendix C). */
 int hp_sequence_scan(const hp_structs* s, const uint64_t* d_ids, int64_t n, const int32_t* d_cand, int32_t k,
@@ -382,7 +391,7 @@ int hp_stream_components(const hp_structs* s, int32_t shard_bits, int32_t window
 const char* hp_last_error(void);
 
 /* Failure-detection hook (no counterpart in the paper).  Every wait of the
- * map kernel and of the tcgen05 GEMM on a shared-memory barrier is bounded:
+ * map kernel, the tensor-core scan and the tcgen05 GEMM on a shared-memory barrier is bounded:
  * after a number of polls it gives up, the kernel records the timeout in its
  * device error word, stops, waits (with a fixed bound of its own) for the
  * copies and tensor-core operations it still has in flight, and returns, and
@@ -390,7 +399,8 @@ const char* hp_last_error(void);
  * hp_autotune) or hp_mlp_status does.  This call sets the poll limit of those
  * waits for every later launch in the process: polls >= 0 sets it (0 gives
  * up at the first check, which lets a test see the timeout path end in
- * HP_ETIMEOUT with the context still usable), polls < 0 restores each
+ * HP_ETIMEOUT with the context still usable; hp_sequence_scan then scores the
+ * sequences without the tensor cores and stays exact), polls < 0 restores each
  * kernel's built-in limit.  The exit drains keep their fixed limit.  It is a
  * process-wide setting for tests: launches made while it is lowered fail.
  * Graph plans keep the limit they were created with.  Always HP_OK. */
