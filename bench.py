@@ -804,7 +804,7 @@ def main():
         "map_performed_evals": performed,
         "tile_cfg": {"reg_bits": tile_cfg[0], "tile": tile_cfg[1]},
         "fold_fraction": float(1.0 - hist[S] / nseq),
-        "gpu_launches": args.steps * (8 + 1 + max(0, -(-(N - 13) // 8))),
+        "gpu_launches": args.steps * (7 + 2 * max(0, -(-(N - 13) // 8))),
         "e2e": {"value": world * evals_step / (e2e_ms * 1e-3), "unit": "evals/s", "h2d_bytes_per_step": 0,
                 "d2h_bytes_per_step": int(d2h),
                 "note": "public Python API; each step's map, labels and reductions copied to pinned host memory inside "
