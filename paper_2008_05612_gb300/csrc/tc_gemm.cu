@@ -324,9 +324,12 @@ __device__ __forceinline__ void topk_chunk(uint32_t (&v)[32], const float* bias,
         for (int e = 0; e < KT; e++) tie |= cv == bv[e];
         if (!tie) {
           if (cv > bv[KT - 1]) {
+            // from the entry it takes the place of on, the list moves down by one: entries that it
+            // displaces may equal the next ones and keep their order
+            bool take = false;
 #pragma unroll
             for (int e = 0; e < KT; e++) {
-              const bool take = cv > bv[e];
+              take = take || cv > bv[e];
               const float tv = bv[e];
               const int ti = bi[e];
               bv[e] = take ? cv : bv[e];
