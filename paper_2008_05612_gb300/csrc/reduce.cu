@@ -232,7 +232,12 @@ enum FlipWork { kRobustness, kPhi, kJoinFirst, kJoin };
 // 247 us) with the longer runs of contiguous ids.
 __host__ __device__ constexpr int block_bits(int work) { return work == kPhi ? kRobTileBits - 1 : kRobTileBits; }
 
-template <int WORK>
+// SHARE (networks of maps below 2^21 ids): a block of 2^9 ids lists one or two times 32, and one warp would
+// join all their pairs one round after another; there the warps share the bits.  Networks of 2^14 ids at the
+// 3x3x3 density 65 -> 60 us, of 2^16 72 -> 68 (whole calls; one id at a time through global labels took 56
+// and 62, but 143 against 123 for the 2^20 ids of 4x5).  In blocks of 2^13, where every warp has ids, the
+// shorter loop is faster: 2^25 ids 617 against 639 us.
+template <int WORK, bool SHARE = false>
 __global__ void __launch_bounds__(kRobThreads) flip_pass(const int32_t* __restrict__ phen, int S, const RobPass P,
                                                                unsigned long long nblocks, int replicas,
                                                                unsigned long long* __restrict__ neutral_rep,
@@ -373,12 +378,15 @@ __global__ void __launch_bounds__(kRobThreads) flip_pass(const int32_t* __restri
       // each warp collects its pairs and joins 32 at a time.  In shared memory the pairs are of this
       // block; across blocks they are global ids and wait for the warp's next ones.
       const uint32_t lt = (1u << lane) - 1u;
-      for (unsigned f0 = threadIdx.x - lane; f0 < n; f0 += blockDim.x) {
+      constexpr unsigned kWarps = kRobThreads / 32;
+      const unsigned warp = threadIdx.x >> 5, groups = (n + 31) / 32;
+      const unsigned share = SHARE && groups && groups < kWarps ? kWarps / groups : 1u;  // warps per 32 ids
+      for (unsigned f0 = 32 * (warp / share); f0 < n; f0 += share > 1 ? n : blockDim.x) {
         const bool have = f0 + lane < n;
         const unsigned idx = have ? list[f0 + lane] : 0u;
         const int32_t p = tile[idx];
         const uint32_t id = WORK == kJoinFirst ? idx : (uint32_t)(base + hoff[idx >> c] + (idx & cmask));
-        for (int t = 0; t < nbits; t++) {
+        for (int t = (int)(warp % share); t < nbits; t += (int)share) {
           const unsigned other = idx ^ (1u << (bit0 + t));
           const bool hit = have && other > idx && tile[other] == p;  // each pair once, from its smaller id
           const uint32_t m = __ballot_sync(0xFFFFFFFFu, hit);
@@ -589,6 +597,7 @@ namespace hp {
 // CTAs of a pass: as many as are resident (they walk the blocks), at most one per block.
 template <class Kernel>
 unsigned pass_grid(Kernel kernel, size_t smem, unsigned long long blocks) {
+  if (blocks <= (unsigned long long)sm_count()) return (unsigned)blocks;
   int per_sm = 0;
   if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kernel, kRobThreads, smem) != cudaSuccess || per_sm < 1) per_sm = 1;
   return (unsigned)std::min<unsigned long long>(blocks, (unsigned long long)sm_count() * per_sm);
@@ -682,16 +691,17 @@ extern "C" int hp_neutral_components(const int32_t* d_phen, int32_t N, int32_t S
   const unsigned long long total = 1ull << N, blocks = total >> hp::flip_block_bits(N, kRobTileBits);
   const size_t smem = 2 * (sizeof(int32_t) << kRobTileBits) + (sizeof(uint16_t) << kRobTileBits);
   const size_t smem1 = smem + (sizeof(uint16_t) << kRobTileBits);  // and the block's parents
-  e = cudaFuncSetAttribute(flip_pass<kJoinFirst>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem1);
-  if (e == cudaSuccess) e = cudaFuncSetAttribute(flip_pass<kJoin>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+  const bool small = hp::flip_block_bits(N, kRobTileBits) < kRobTileBits;
+  const auto first = small ? flip_pass<kJoinFirst, true> : flip_pass<kJoinFirst>;
+  const auto later = small ? flip_pass<kJoin, true> : flip_pass<kJoin>;
+  e = cudaFuncSetAttribute(first, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem1);
+  if (e == cudaSuccess) e = cudaFuncSetAttribute(later, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
   if (e == cudaSuccess) {
     for (const RobPass& p : hp::flip_passes(N, kRobTileBits)) {
-      if (p.first)
-        flip_pass<kJoinFirst><<<hp::pass_grid(flip_pass<kJoinFirst>, smem1, blocks), kRobThreads, smem1, st>>>(d_phen, S, p, blocks, 1, nullptr, nullptr, nullptr, err,
-                                                                  hp::PhiTable{}, d_label);
-      else
-        flip_pass<kJoin><<<hp::pass_grid(flip_pass<kJoin>, smem, blocks), kRobThreads, smem, st>>>(d_phen, S, p, blocks, 1, nullptr, nullptr, nullptr, err,
-                                                            hp::PhiTable{}, d_label);
+      const auto pass = p.first ? first : later;
+      const size_t bytes = p.first ? smem1 : smem;
+      pass<<<hp::pass_grid(pass, bytes, blocks), kRobThreads, bytes, st>>>(d_phen, S, p, blocks, 1, nullptr, nullptr, nullptr,
+                                                                          err, hp::PhiTable{}, d_label);
     }
     const unsigned grid = (unsigned)std::min<unsigned long long>((total + 1023) / 1024, (unsigned long long)sm_count() * 16);
     cc_finish<<<grid, 256, 0, st>>>(d_phen, total, d_label, reinterpret_cast<unsigned long long*>(d_ncomp));
