@@ -38,7 +38,7 @@ struct DevTables {
   // tensor-core scan (built on first use): 0/1 contact rows over the pairs that occur, in slab order
   uint8_t* tc_tab = nullptr;
   uint16_t* tc_pairs = nullptr;    // 32 tc_nk pairs: even index | odd index << 8
-  int tc_nk = 0, tc_ntiles = 0;    // slabs of 32 pairs (0: not built, -1: no room), tiles of 256
+  int tc_nk = 0, tc_ntiles = 0;    // slabs of 32 pairs (0: not built, -1: too large), tiles of 256
   // class -> first conformation index and number of conformations (built on first use)
   int32_t* class_first = nullptr;
   int32_t* class_nconf = nullptr;

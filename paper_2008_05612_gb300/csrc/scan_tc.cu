@@ -31,6 +31,8 @@
 #include <algorithm>
 #include <climits>
 #include <cstring>
+#include <memory>
+#include <new>
 #include <string>
 #include <vector>
 
@@ -480,7 +482,9 @@ __global__ void __launch_bounds__(256) scan_tc_resolve(const ResolveParams p) {
   }
 }
 
-// The pairs in contact in some conformation, and the conformations' 0/1 rows over them in slab order.
+// The pairs in contact in some conformation, and the conformations' 0/1 rows over them in slab order.  A
+// table above kMaxTable is never built (tc_nk -1); one that finds no room now is tried again by the next
+// call (tc_nk stays 0), and this call's ids go to the caller's other kernel.
 int scan_tc_tables(const hp_structs* cs, hp::DevTables** out) {
   hp::DevTables* dt = nullptr;
   const int rc = hp::device_tables(cs, &dt);
@@ -511,26 +515,34 @@ int scan_tc_tables(const hp_structs* cs, hp::DevTables** out) {
     dt->tc_nk = -1;
     return HP_OK;
   }
-  std::vector<uint8_t> tab(bytes, 0);
+  // the device's memory first: a call that gets none leaves tc_nk at 0 and costs no more than this
+  uint8_t* d_tab = nullptr;
+  uint16_t* d_pairs = nullptr;
+  cudaError_t e = cudaMalloc(&d_tab, bytes);
+  if (e == cudaSuccess) e = cudaMalloc(&d_pairs, pairs.size() * 2);
+  const std::unique_ptr<uint8_t[]> tab(e == cudaSuccess ? new (std::nothrow) uint8_t[bytes]() : nullptr);
+  if (!tab) {
+    cudaFree(d_tab);
+    cudaFree(d_pairs);
+    cudaGetLastError();
+    return HP_OK;
+  }
   auto at = [&](size_t conf, int k) -> uint8_t& {
     const size_t t = conf / kTile, r = conf % kTile;
     return tab[(t * nk + k / 32) * kSlabB + (r / 8) * 256 + ((k / 16) & 1) * 128 + (r % 8) * 16 + k % 16];
   };
   for (size_t c = 0; c < nc; c++) at(c / s->C, col[pair_of(c)]) = (uint8_t)kF1;
   for (size_t c = (size_t)s->S_dir; c < (size_t)ntiles * kTile; c++) at(c, cpad) = (uint8_t)kF448;
-  cudaError_t e = cudaMalloc(&dt->tc_tab, bytes);
-  if (e == cudaSuccess) e = cudaMalloc(&dt->tc_pairs, pairs.size() * 2);
-  if (e == cudaSuccess) e = cudaMemcpy(dt->tc_tab, tab.data(), bytes, cudaMemcpyHostToDevice);
-  if (e == cudaSuccess) e = cudaMemcpy(dt->tc_pairs, pairs.data(), pairs.size() * 2, cudaMemcpyHostToDevice);
+  e = cudaMemcpy(d_tab, tab.get(), bytes, cudaMemcpyHostToDevice);
+  if (e == cudaSuccess) e = cudaMemcpy(d_pairs, pairs.data(), pairs.size() * 2, cudaMemcpyHostToDevice);
   if (e != cudaSuccess) {
-    cudaFree(dt->tc_tab);
-    cudaFree(dt->tc_pairs);
-    dt->tc_tab = nullptr;
-    dt->tc_pairs = nullptr;
+    cudaFree(d_tab);
+    cudaFree(d_pairs);
     cudaGetLastError();
-    dt->tc_nk = -1;  // no room for the table: the warp scan serves this device
     return HP_OK;
   }
+  dt->tc_tab = d_tab;
+  dt->tc_pairs = d_pairs;
   dt->tc_nk = nk;
   dt->tc_ntiles = ntiles;
   return HP_OK;
@@ -548,7 +560,7 @@ int scan_tc(const hp_structs* s, const ScanTc& a, cudaStream_t st, long long* do
   DevTables* dt = nullptr;
   int rc = scan_tc_tables(s, &dt);
   if (rc != HP_OK) return rc;
-  if (dt->tc_nk < 0) return HP_OK;
+  if (dt->tc_nk <= 0) return HP_OK;
   int dev = 0, sms = 0;
   cudaGetDevice(&dev);
   cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
