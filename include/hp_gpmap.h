@@ -170,8 +170,7 @@ void hp_batch_plan_free(hp_batch_plan* plan);
 
 /* Ground state of an arbitrary list of sequence ids (e.g. a seeded sample,
  * the paper's sampling mode of Table 3).  Every conformation is scored on the
- * tensor cores (stream-ordered scratch of at most 27 MB; a capture records
- * it), except in small scans (at most 1,024 conformations and n times these at
+ * tensor cores (stream-ordered scratch of at most 27 MB), except in small scans (at most 1,024 conformations and n times these at
  * most 2^22), where its table or scratch does not fit, and in calls with both
  * d_cand and d_counters: these run one warp per sequence, with optional exact
  * bound pruning seeded by candidate conformations (the learned proposal).  With A_s(h) = sum_i h_i c_i(s) and B the HH-contact count,
@@ -188,8 +187,13 @@ void hp_batch_plan_free(hp_batch_plan* plan);
  *   d_counters: device uint64[2] (or NULL): conformations evaluated exactly
  *               and group bounds evaluated are ADDED to [0] and [1] (n times
  *               the conformations and 0 without candidates).
- * Stream-ordered; does not synchronise.  No counterpart in the paper beyond
- * its sampled kernel (Appendix C). */
+ * Stream-ordered; does not synchronise.  May be captured once the library has
+ * been used on the device: the capture records kernels alone, any number of
+ * instances and parent graphs may hold it, and all of them must be gone
+ * before the library is freed.  A captured tensor-core scan holds 27 MB of
+ * scratch per 2^19 ids (or less for fewer) until its graph and instances are
+ * destroyed; the library keeps it for later captures until hp_structs_free.
+ * No counterpart in the paper beyond its sampled kernel (Appendix C). */
 int hp_sequence_scan(const hp_structs* s, const uint64_t* d_ids, int64_t n, const int32_t* d_cand, int32_t k,
                      int32_t* d_phen, int32_t* d_aux, uint64_t* d_counters, void* stream);
 

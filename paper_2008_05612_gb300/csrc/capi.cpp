@@ -30,6 +30,32 @@ long long wait_limit(long long dflt) {
   return v < 0 ? dflt : v;
 }
 
+TableUpload::TableUpload() {
+  cudaThreadExchangeStreamCaptureMode(&mode_);
+  err_ = cudaStreamCreateWithFlags(&st_, cudaStreamNonBlocking);
+}
+
+TableUpload::~TableUpload() {
+  if (st_) cudaStreamDestroy(st_);
+  cudaThreadExchangeStreamCaptureMode(&mode_);
+}
+
+cudaError_t TableUpload::alloc(void** d, size_t bytes) {
+  if (err_ == cudaSuccess) err_ = cudaMalloc(d, bytes);
+  return err_;
+}
+
+cudaError_t TableUpload::copy(void* d, const void* h, size_t bytes) {
+  if (err_ == cudaSuccess) err_ = cudaMemcpyAsync(d, h, bytes, cudaMemcpyHostToDevice, st_);
+  return err_;
+}
+
+cudaError_t TableUpload::finish() {
+  const cudaError_t e = st_ ? cudaStreamSynchronize(st_) : cudaSuccess;
+  if (err_ == cudaSuccess) err_ = e;
+  return err_;
+}
+
 int device_tables(const hp_structs* cs, DevTables** out) {
   hp_structs* s = const_cast<hp_structs*>(cs);
   int dev = 0;
@@ -101,6 +127,14 @@ extern "C" void hp_structs_free(hp_structs* s) {
       if (t->scan_midx) cudaFree(t->scan_midx);
       if (t->tc_tab) cudaFree(t->tc_tab);
       if (t->tc_pairs) cudaFree(t->tc_pairs);
+      if (t->graph_scratch) {
+        std::vector<hp::GraphScratch::Block> blocks;
+        {
+          std::lock_guard<std::mutex> lock(t->graph_scratch->mu);
+          blocks.swap(t->graph_scratch->blocks);
+        }
+        for (const hp::GraphScratch::Block& b : blocks) cudaFree(b.p);
+      }
       if (t->class_first) cudaFree(t->class_first);
       if (t->class_nconf) cudaFree(t->class_nconf);
       if (t->half_otab) cudaFree(t->half_otab);

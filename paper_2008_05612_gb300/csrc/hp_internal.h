@@ -4,6 +4,7 @@
 #include <cuda_runtime.h>
 
 #include <cstdint>
+#include <memory>
 #include <mutex>
 #include <string>
 #include <vector>
@@ -19,6 +20,39 @@ constexpr int kMaxSym = 48;     // order of the cube's symmetry group
 // Sets the thread-local error text and returns `code`.
 int fail(int code, const std::string& msg);
 int cuda_fail(int err, const char* what);  // err is a cudaError_t
+
+// Scratch of captured scans: a block is its graph's until the graph and its instances are gone, then the
+// next capture's; freed with the library.
+struct GraphScratch {
+  struct Block {
+    void* p;
+    size_t bytes;
+    bool used;
+  };
+  std::mutex mu;
+  std::vector<Block> blocks;
+};
+
+// Allocation and upload of a library's tables on their first use, which may lie inside a stream capture:
+// meanwhile this thread's capture mode is relaxed, and the copies run on a stream of their own.  Keeps the
+// first error.
+class TableUpload {
+ public:
+  TableUpload();
+  ~TableUpload();
+  cudaError_t alloc(void** d, size_t bytes);
+  cudaError_t copy(void* d, const void* h, size_t bytes);  // h stays until finish()
+  template <class T>
+  void table(T** d, const std::vector<T>& h) {
+    if (alloc(reinterpret_cast<void**>(d), h.size() * sizeof(T)) == cudaSuccess) copy(*d, h.data(), h.size() * sizeof(T));
+  }
+  cudaError_t finish();  // waits for the copies
+
+ private:
+  cudaStreamCaptureMode mode_ = cudaStreamCaptureModeRelaxed;
+  cudaStream_t st_ = nullptr;
+  cudaError_t err_ = cudaSuccess;
+};
 
 // Per-device copy of a fold library's kernel tables.
 struct DevTables {
@@ -38,6 +72,7 @@ struct DevTables {
   // tensor-core scan (built on first use): 0/1 contact rows over the pairs that occur, in slab order
   uint8_t* tc_tab = nullptr;
   uint16_t* tc_pairs = nullptr;    // 32 tc_nk pairs: even index | odd index << 8
+  std::shared_ptr<GraphScratch> graph_scratch;
   int tc_nk = 0, tc_ntiles = 0;    // slabs of 32 pairs (0: not built, -1: too large), tiles of 256
   // class -> first conformation index and number of conformations (built on first use)
   int32_t* class_first = nullptr;

@@ -518,9 +518,10 @@ int scan_tc_tables(const hp_structs* cs, hp::DevTables** out) {
   // the device's memory first: a call that gets none leaves tc_nk at 0 and costs no more than this
   uint8_t* d_tab = nullptr;
   uint16_t* d_pairs = nullptr;
-  cudaError_t e = cudaMalloc(&d_tab, bytes);
-  if (e == cudaSuccess) e = cudaMalloc(&d_pairs, pairs.size() * 2);
-  const std::unique_ptr<uint8_t[]> tab(e == cudaSuccess ? new (std::nothrow) uint8_t[bytes]() : nullptr);
+  hp::TableUpload up;
+  up.alloc(reinterpret_cast<void**>(&d_tab), bytes);
+  const cudaError_t got = up.alloc(reinterpret_cast<void**>(&d_pairs), pairs.size() * 2);
+  const std::unique_ptr<uint8_t[]> tab(got == cudaSuccess ? new (std::nothrow) uint8_t[bytes]() : nullptr);
   if (!tab) {
     cudaFree(d_tab);
     cudaFree(d_pairs);
@@ -533,9 +534,9 @@ int scan_tc_tables(const hp_structs* cs, hp::DevTables** out) {
   };
   for (size_t c = 0; c < nc; c++) at(c / s->C, col[pair_of(c)]) = (uint8_t)kF1;
   for (size_t c = (size_t)s->S_dir; c < (size_t)ntiles * kTile; c++) at(c, cpad) = (uint8_t)kF448;
-  e = cudaMemcpy(d_tab, tab.get(), bytes, cudaMemcpyHostToDevice);
-  if (e == cudaSuccess) e = cudaMemcpy(d_pairs, pairs.data(), pairs.size() * 2, cudaMemcpyHostToDevice);
-  if (e != cudaSuccess) {
+  up.copy(d_tab, tab.get(), bytes);
+  up.copy(d_pairs, pairs.data(), pairs.size() * 2);
+  if (up.finish() != cudaSuccess) {
     cudaFree(d_tab);
     cudaFree(d_pairs);
     cudaGetLastError();
@@ -548,13 +549,77 @@ int scan_tc_tables(const hp_structs* cs, hp::DevTables** out) {
   return HP_OK;
 }
 
+struct ScratchLease {
+  std::shared_ptr<hp::GraphScratch> pool;
+  size_t block;
+};
+
+void CUDART_CB end_lease(void* p) {  // (may run on a thread of the driver: no CUDA calls)
+  ScratchLease* l = static_cast<ScratchLease*>(p);
+  {
+    std::lock_guard<std::mutex> lock(l->pool->mu);
+    if (l->block < l->pool->blocks.size()) l->pool->blocks[l->block].used = false;  // (empty: the library is gone)
+  }
+  delete l;
+}
+
+// Scratch for a scan that is being captured into graph; NULL where there is none.  Stream-ordered memory would
+// put memory nodes into the graph, of which only one instance may then exist and which no other graph
+// may hold; this block is the graph's by reference instead (a user object, which its instances and
+// clones hold too).
+char* graph_scratch(hp_structs* s, hp::DevTables* dt, cudaGraph_t graph, size_t bytes) try {
+  {
+    std::lock_guard<std::mutex> lock(s->mu);
+    if (!dt->graph_scratch) dt->graph_scratch = std::make_shared<hp::GraphScratch>();
+  }
+  // no CUDA call is made under the pool's lock, which end_lease takes
+  hp::GraphScratch& pool = *dt->graph_scratch;
+  std::unique_ptr<ScratchLease> lease(new ScratchLease{dt->graph_scratch, 0});
+  void* p = nullptr;
+  {
+    std::lock_guard<std::mutex> lock(pool.mu);
+    std::vector<hp::GraphScratch::Block>& b = pool.blocks;
+    size_t best = b.size();  // the smallest free block that is large enough, or else a place without memory
+    for (size_t i = 0; i < b.size(); i++)
+      if (!b[i].used && b[i].bytes >= bytes && (best == b.size() || b[i].bytes < b[best].bytes)) best = i;
+    for (size_t i = 0; i < b.size() && best == b.size(); i++)
+      if (!b[i].used && !b[i].p) best = i;
+    if (best == b.size()) b.push_back({nullptr, 0, false});
+    b[best].used = true;
+    p = b[best].p;
+    lease->block = best;
+  }
+  bool ok = p != nullptr;
+  if (!ok) {
+    hp::TableUpload relaxed;
+    ok = relaxed.alloc(&p, bytes) == cudaSuccess;
+    std::lock_guard<std::mutex> lock(pool.mu);
+    pool.blocks[lease->block].p = ok ? p : nullptr;
+    pool.blocks[lease->block].bytes = ok ? bytes : 0;
+  }
+  cudaUserObject_t obj = nullptr;
+  ok = ok && cudaUserObjectCreate(&obj, lease.get(), end_lease, 1, cudaUserObjectNoDestructorSync) == cudaSuccess;
+  if (!ok) {
+    cudaGetLastError();
+    end_lease(lease.release());
+    return nullptr;
+  }
+  lease.release();  // now the object's
+  if (cudaGraphRetainUserObject(graph, obj, 1, cudaGraphUserObjectMove) != cudaSuccess) {
+    cudaGetLastError();
+    cudaUserObjectRelease(obj, 1);
+    return nullptr;
+  }
+  return static_cast<char*>(p);
+} catch (const std::bad_alloc&) {
+  return nullptr;
+}
+
 }  // namespace
 
 namespace hp {
 
-// *done = 0: the caller's other kernel has to take the ids (the table or the scratch does not fit).  The
-// scratch is stream-ordered, so a capture records it with the two kernels (and, as for every scan, needs
-// the tables to be there from an earlier call).
+// *done = 0: the caller's other kernel has to take the ids (the table or the scratch does not fit).
 int scan_tc(const hp_structs* s, const ScanTc& a, cudaStream_t st, long long* done) {
   *done = 0;
   DevTables* dt = nullptr;
@@ -586,11 +651,19 @@ int scan_tc(const hp_structs* s, const ScanTc& a, cudaStream_t st, long long* do
   const long long chunk = std::min<long long>(a.n, kChunk);
   const long long blocks = (chunk + kBlock - 1) / kBlock;
   const size_t part = sizeof(float) * 3 * kParts * kBlock * (size_t)(blocks + sms);
+  const size_t bytes = (part + sizeof(unsigned) * sms + 255) / 256 * 256;
+  cudaStreamCaptureStatus capture = cudaStreamCaptureStatusNone;
+  cudaGraph_t graph = nullptr;
+  if (cudaStreamGetCaptureInfo(st, &capture, nullptr, &graph) != cudaSuccess) cudaGetLastError();
+  const bool captured = capture == cudaStreamCaptureStatusActive;
   char* scratch = nullptr;
-  if (cudaMallocAsync(reinterpret_cast<void**>(&scratch), part + sizeof(unsigned) * sms, st) != cudaSuccess) {
+  if (captured) {  // each launch its own part: instances of the graph may run side by side
+    scratch = graph_scratch(const_cast<hp_structs*>(s), dt, graph, bytes * (size_t)((a.n + chunk - 1) / chunk));
+  } else if (cudaMallocAsync(reinterpret_cast<void**>(&scratch), bytes, st) != cudaSuccess) {
     cudaGetLastError();
-    return HP_OK;
+    scratch = nullptr;
   }
+  if (!scratch) return HP_OK;
   p.part = reinterpret_cast<float*>(scratch);
   p.status = reinterpret_cast<unsigned*>(scratch + part);
   for (long long off = 0; off < a.n && rc == HP_OK; off += chunk) {
@@ -619,8 +692,12 @@ int scan_tc(const hp_structs* s, const ScanTc& a, cudaStream_t st, long long* do
     scan_tc_resolve<<<(unsigned)((p.n + 7) / 8), 256, 0, st>>>(r);
     e = cudaGetLastError();
     if (e != cudaSuccess) rc = cuda_fail(e, "tensor-core scan: launch");
+    if (captured) {
+      p.part = reinterpret_cast<float*>(reinterpret_cast<char*>(p.part) + bytes);
+      p.status = reinterpret_cast<unsigned*>(reinterpret_cast<char*>(p.status) + bytes);
+    }
   }
-  cudaFreeAsync(scratch, st);
+  if (!captured) cudaFreeAsync(scratch, st);
   if (rc == HP_OK) *done = a.n;
   return rc;
 }

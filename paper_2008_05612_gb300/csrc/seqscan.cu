@@ -389,20 +389,15 @@ int scan_tables(const hp_structs* cs, DevTables** out) {
     }
     midx[j] = order[j];
   }
-  cudaError_t e = cudaMalloc(&dt->scan_gcnt, gcnt.size() * 4);
-  if (e == cudaSuccess) e = cudaMalloc(&dt->scan_ccnt, ccnt.size() * 4);
-  if (e == cudaSuccess) e = cudaMemcpy(dt->scan_ccnt, ccnt.data(), ccnt.size() * 4, cudaMemcpyHostToDevice);
-  if (e == cudaSuccess) e = cudaMalloc(&dt->scan_cl1, cl1.size() * 4);
-  if (e == cudaSuccess) e = cudaMemcpy(dt->scan_cl1, cl1.data(), cl1.size() * 4, cudaMemcpyHostToDevice);
-  if (e == cudaSuccess) e = cudaMalloc(&dt->scan_gbeg, gbeg.size() * 4);
-  if (e == cudaSuccess) e = cudaMalloc(&dt->scan_mcnt, mcnt.size() * 4);
-  if (e == cudaSuccess) e = cudaMalloc(&dt->scan_mmask, mmask.size() * 4);
-  if (e == cudaSuccess) e = cudaMalloc(&dt->scan_midx, midx.size() * 4);
-  if (e == cudaSuccess) e = cudaMemcpy(dt->scan_gcnt, gcnt.data(), gcnt.size() * 4, cudaMemcpyHostToDevice);
-  if (e == cudaSuccess) e = cudaMemcpy(dt->scan_gbeg, gbeg.data(), gbeg.size() * 4, cudaMemcpyHostToDevice);
-  if (e == cudaSuccess) e = cudaMemcpy(dt->scan_mcnt, mcnt.data(), mcnt.size() * 4, cudaMemcpyHostToDevice);
-  if (e == cudaSuccess) e = cudaMemcpy(dt->scan_mmask, mmask.data(), mmask.size() * 4, cudaMemcpyHostToDevice);
-  if (e == cudaSuccess) e = cudaMemcpy(dt->scan_midx, midx.data(), midx.size() * 4, cudaMemcpyHostToDevice);
+  TableUpload up;
+  up.table(&dt->scan_gcnt, gcnt);
+  up.table(&dt->scan_ccnt, ccnt);
+  up.table(&dt->scan_cl1, cl1);
+  up.table(&dt->scan_gbeg, gbeg);
+  up.table(&dt->scan_mcnt, mcnt);
+  up.table(&dt->scan_mmask, mmask);
+  up.table(&dt->scan_midx, midx);
+  const cudaError_t e = up.finish();
   if (e != cudaSuccess) {
     cudaFree(dt->scan_gcnt);
     cudaFree(dt->scan_ccnt);

@@ -1,6 +1,7 @@
 """Scans of a list of ids in CUDA graphs and around them: which kernels a capture records, what may be done with its
 graph, and that a table or scratch that could not be had once is had by the next call."""
 import ctypes
+import time
 
 import numpy as np
 import pytest
@@ -107,3 +108,89 @@ def test_a_table_that_found_no_memory_is_built_by_a_later_call(hp):
     assert later.error is None
     assert later.nodes().count(KERNEL_NODE) == 2  # the scan and what resolves its ties, not the warp scan
     later.destroy()
+
+
+@pytest.mark.parametrize("dims", [(5, 5), (3, 3, 3)])
+@pytest.mark.parametrize("counted", [False, True])
+def test_a_scan_makes_every_later_scan_capturable(hp, dims, counted):
+    """The tensor-core scan and the warp scan have tables of their own; a capture of one after only the other has run."""
+    s, ref = hp.Structs(dims), hp.Structs(dims)
+    ids = ids_of(s.N, 5000, 11)
+    cand = torch.zeros((5000, 1), dtype=torch.int32, device="cuda")
+    cnt = torch.zeros(2, dtype=torch.int64, device="cuda")
+    plain = lambda h: hp.sequence_scan(h, ids, aux=True)
+    pruned = lambda h: hp.sequence_scan(h, ids, cand=cand, aux=True, counters=cnt)
+    first, then = (pruned, plain) if not counted else (plain, pruned)
+    want = plain(ref)
+    first(s)
+    c = Capture(5000, lambda: then(s))
+    assert c.error is None, c.error
+    for t in c.out:
+        t.zero_()
+    torch.cuda.synchronize()
+    rc, x = c.instance()
+    assert rc == 0
+    c.launch(x)
+    torch.cuda.synchronize()
+    assert all(torch.equal(a, b) for a, b in zip(c.out, want))
+    assert c.rt.cudaGraphExecDestroy(x) == 0
+    c.destroy()
+
+
+@pytest.mark.parametrize("n", [700, (1 << 19) + 131])  # one launch and two
+def test_a_captured_scan_is_kernels_alone(hp, n):
+    """So its graph may have two instances, side by side on two streams, and be a node of another graph."""
+    s = hp.Structs((5, 5))
+    ids = ids_of(25, n, 13)
+    want = hp.sequence_scan(s, ids)
+    c = Capture(n, lambda: hp.sequence_scan(s, ids))
+    assert c.error is None, c.error
+    assert set(c.nodes()) == {KERNEL_NODE}
+    other, parent, node = torch.cuda.Stream(), ctypes.c_void_p(), ctypes.c_void_p()
+    assert c.rt.cudaGraphCreate(ctypes.byref(parent), 0) == 0
+    assert c.rt.cudaGraphAddChildGraphNode(ctypes.byref(node), parent, None, ctypes.c_size_t(0), c.graph) == 0
+    (rc0, x0), (rc1, x1), (rc2, x2) = c.instance(), c.instance(), c.instance(parent)
+    assert (rc0, rc1, rc2) == (0, 0, 0)
+    c.destroy()  # the instances keep the scratch
+    again = Capture(n, lambda: hp.sequence_scan(s, ids ^ 1))
+    assert again.error is None
+    for use in ([x0, x1], [x2]):
+        c.out.zero_()
+        torch.cuda.synchronize()
+        for _ in range(5):
+            for x, st in zip(use, (c.stream, other)):
+                c.launch(x, st)
+        torch.cuda.synchronize()
+        assert torch.equal(c.out, want)
+    for x in (x0, x1, x2):
+        assert c.rt.cudaGraphExecDestroy(x) == 0
+    assert c.rt.cudaGraphDestroy(parent) == 0
+    again.destroy()
+
+
+def test_captures_share_scratch_over_time_and_the_library_gives_it_back(hp):
+    s = hp.Structs((5, 5))
+    n = 1 << 19
+    ids = ids_of(25, n, 17)
+    hp.sequence_scan(s, ids)
+    torch.cuda.synchronize()
+
+    def one():
+        c = Capture(n, lambda: hp.sequence_scan(s, ids))
+        assert c.error is None
+        rc, x = c.instance()
+        assert rc == 0
+        c.launch(x)
+        torch.cuda.synchronize()
+        assert c.rt.cudaGraphExecDestroy(x) == 0
+        c.destroy()
+        del c
+        torch.cuda.empty_cache()
+        time.sleep(0.02)  # the driver may end the scratch's use a little later
+        return torch.cuda.mem_get_info()[0]
+
+    first = one()
+    free = [one() for _ in range(12)]
+    assert first - min(free) < 3 * (28 << 20)  # not 12 blocks of 27 MB
+    del s
+    assert torch.cuda.mem_get_info()[0] >= min(free) + (27 << 20) - (2 << 20)
