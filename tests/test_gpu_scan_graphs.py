@@ -26,12 +26,16 @@ def hp():
     return m
 
 
+def runtime():
+    """The CUDA runtime that torch has loaded."""
+    return ctypes.CDLL("libcudart.so.%s" % torch.version.cuda.split(".")[0])
+
+
 class Capture:
-    """call() captured on a stream of its own, through the CUDA runtime that torch has loaded; its outputs are of
-    n ids."""
+    """call() captured on a stream of its own; its outputs are of n ids."""
 
     def __init__(self, n, call):
-        self.rt = ctypes.CDLL("libcudart.so.%s" % torch.version.cuda.split(".")[0])
+        self.rt = runtime()
         self.stream = torch.cuda.Stream()
         self.graph = ctypes.c_void_p()
         self.error = None
@@ -91,18 +95,21 @@ def test_a_table_that_found_no_memory_is_built_by_a_later_call(hp):
     s = hp.Structs((3, 3, 3))
     ids = ids_of(27, 64, 3)
     want = warp_scan(hp, s, ids)
+    rt = runtime()
     hog, size = [], torch.cuda.mem_get_info()[0]
-    while size >= 1 << 21:  # all but a few MB of the device
-        try:
-            hog.append(torch.empty(size, dtype=torch.uint8, device="cuda"))
-        except torch.OutOfMemoryError:
+    while size >= 1 << 21:  # all but a few MB of the device (torch's allocator takes 20 MB at a time)
+        p = ctypes.c_void_p()
+        if rt.cudaMalloc(ctypes.byref(p), ctypes.c_size_t(size)) == 0:
+            hog.append(p)
+        else:
+            rt.cudaGetLastError()
             size //= 2
     try:
         assert torch.cuda.mem_get_info()[0] < 1 << 23
         assert torch.equal(hp.sequence_scan(s, ids), want)
     finally:
-        del hog
-        torch.cuda.empty_cache()
+        for p in hog:
+            assert rt.cudaFree(p) == 0
     assert torch.equal(hp.sequence_scan(s, ids), want)
     later = Capture(64, lambda: hp.sequence_scan(s, ids))
     assert later.error is None
