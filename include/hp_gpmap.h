@@ -170,7 +170,7 @@ void hp_batch_plan_free(hp_batch_plan* plan);
 
 /* Ground state of an arbitrary list of sequence ids (e.g. a seeded sample,
  * the paper's sampling mode of Table 3).  Every conformation is scored on the
- * tensor cores (stream-ordered scratch of at most 27 MB), except in small scans (at most 1,024 conformations and n times these at
+ * tensor cores (stream-ordered scratch of at most 27 MB, from a pool that keeps 32 MB per library and device), except in small scans (at most 1,024 conformations and n times these at
  * most 2^22), where its table or scratch does not fit, and in calls with both
  * d_cand and d_counters: these run one warp per sequence, with optional exact
  * bound pruning seeded by candidate conformations (the learned proposal).  With A_s(h) = sum_i h_i c_i(s) and B the HH-contact count,

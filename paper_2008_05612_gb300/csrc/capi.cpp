@@ -127,6 +127,7 @@ extern "C" void hp_structs_free(hp_structs* s) {
       if (t->scan_midx) cudaFree(t->scan_midx);
       if (t->tc_tab) cudaFree(t->tc_tab);
       if (t->tc_pairs) cudaFree(t->tc_pairs);
+      if (t->scan_pool) cudaMemPoolDestroy(t->scan_pool);
       if (t->graph_scratch) {
         std::vector<hp::GraphScratch::Block> blocks;
         {

@@ -73,6 +73,7 @@ struct DevTables {
   uint8_t* tc_tab = nullptr;
   uint16_t* tc_pairs = nullptr;    // 32 tc_nk pairs: even index | odd index << 8
   std::shared_ptr<GraphScratch> graph_scratch;
+  cudaMemPool_t scan_pool = nullptr;  // scratch of its other calls
   int tc_nk = 0, tc_ntiles = 0;    // slabs of 32 pairs (0: not built, -1: too large), tiles of 256
   // class -> first conformation index and number of conformations (built on first use)
   int32_t* class_first = nullptr;

@@ -201,3 +201,24 @@ def test_captures_share_scratch_over_time_and_the_library_gives_it_back(hp):
     assert first - min(free) < 3 * (28 << 20)  # not 12 blocks of 27 MB
     del s
     assert torch.cuda.mem_get_info()[0] >= min(free) + (27 << 20) - (2 << 20)
+
+
+def test_the_library_keeps_one_launch_of_scratch_and_gives_it_back(hp):
+    s = hp.Structs((5, 5))
+    n = 1 << 19
+    ids = ids_of(25, n, 19)
+    want = hp.sequence_scan(s, ids)
+    streams = [torch.cuda.Stream() for _ in range(4)]
+    for _ in range(3):  # scans on several streams take scratch side by side
+        outs = [hp.sequence_scan(s, ids, stream=st) for st in streams]
+        torch.cuda.synchronize()
+        assert all(torch.equal(o, want) for o in outs)
+        held = torch.cuda.mem_get_info()[0]
+    for _ in range(3):
+        hp.sequence_scan(s, ids)
+        torch.cuda.synchronize()
+        assert torch.cuda.mem_get_info()[0] >= held
+    held = torch.cuda.mem_get_info()[0]
+    del s
+    back = torch.cuda.mem_get_info()[0] - held
+    assert (26 << 20) <= back <= (72 << 20)  # 27 MB kept of four times 27, and the tables
