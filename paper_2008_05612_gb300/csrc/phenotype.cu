@@ -1127,12 +1127,17 @@ namespace {
 // odd one, which pays where an aligned block leaves many even residues free: a block of 2^m ids has
 // ceil(m / 2), and a CTA always evaluates 2^roles patterns.  The aligned blocks of a range grow and
 // then shrink, so the blocks of at least 2^m ids are one run; the m with the least estimated time is
-// taken.  Rates measured on 3x3x3, 2x3x4, 6x6 (scores/s): map kernel 3.5e13 with 14 roles, 2.9e13 with 12,
-// 2.15e13 with 11 (2.5e13 with tiles of 128); scan 7.9e-14 s max(1, pairs / 150) conformations + 0.62 ns per id.  2^20 ids of 3x3x3 take 9.0 ms by
-// the scan, and 2^21 8.9 by the map kernel and 18 by the scan.
+// taken.  Rates measured on 3x3x3, 2x3x4, 6x6 with 152 SMs (scores/s): map kernel 3.5e13 with 14 roles,
+// 2.9e13 with 12, 2.15e13 with 11 (2.5e13 with tiles of 128); scan 7.9e-14 s max(1, pairs / 150)
+// conformations + 0.62 ns per id.  2^20 ids of 3x3x3 take 9.0 ms by the scan, and 2^21 8.9 by the map
+// kernel and 18 by the scan.  Thresholds above 1 (14 roles always) are charged the rate at 1.
 void split_range(const hp_structs* s, uint64_t begin, uint64_t count, int gap_threshold, uint64_t* map_begin,
                  uint64_t* map_end) {
-  constexpr double kSms = 152;
+  int dev = 0, n_sms = 0;
+  cudaGetDevice(&dev);
+  cudaDeviceGetAttribute(&n_sms, cudaDevAttrMultiProcessorCount, dev);
+  constexpr double kRateSms = 152;  // the SMs that the rates are of
+  const double sms = n_sms > 0 ? n_sms : kRateSms;
   struct Block {
     uint64_t at;
     int m;
@@ -1146,7 +1151,7 @@ void split_range(const hp_structs* s, uint64_t begin, uint64_t count, int gap_th
     pos += 1ull << m;
   }
   const double pairs = (double)s->NE * s->NO - (s->N - 1);  // pairs that may be in contact
-  const double scan_id = 0.62e-9 + 7.9e-14 * std::max(1.0, pairs / 150.0) * s->S_dir;
+  const double scan_id = (0.62e-9 + 7.9e-14 * std::max(1.0, pairs / 150.0) * s->S_dir) * kRateSms / sms;
   double best = 40e-6 + count * scan_id;  // no block to the map kernel
   *map_begin = *map_end = begin;
   for (int mmin = 0; mmin < 63; mmin++) {
@@ -1169,10 +1174,12 @@ void split_range(const hp_structs* s, uint64_t begin, uint64_t count, int gap_th
         const int ne = std::min((b.m + 1) / 2, s->NE);
         items += std::ldexp(half ? 0.51 : 1.0, b.m - std::min(ne, roles));
       }
+    // CTAs of an SM.  The 11-role shape with tiles of 128 has two; as four, so that fewer than two rounds of
+    // items cost two, which they do (2^19 ids of 3x3x3: 5.4 ms by the map kernel, 4.5 by the scan).
     const double ctas = roles == 14 ? 1 : roles == 12 ? 2 : 4;
     const double rate = roles == 14 ? 3.5e13 : roles == 12 ? 2.9e13 : t == 128 ? 2.5e13 : 2.15e13;
-    const double item = std::ldexp((double)s->S_dir, roles) * kSms * ctas / rate + 20e-6;
-    const double waves = std::max(1.0, items / (kSms * ctas));
+    const double item = std::ldexp((double)s->S_dir, roles) * kRateSms * ctas / rate + 20e-6;
+    const double waves = std::max(1.0, items / (sms * ctas));
     const uint64_t rest = count - ids;
     const double cost = 25e-6 + waves * item + (rest ? 40e-6 + rest * scan_id : 0.0);
     if (cost < best) {
