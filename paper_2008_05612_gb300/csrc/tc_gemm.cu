@@ -323,20 +323,12 @@ __device__ __forceinline__ void topk_chunk(uint32_t (&v)[32], const float* bias,
 #pragma unroll
         for (int e = 0; e < KT; e++) tie |= cv == bv[e];
         if (!tie) {
-          if (cv > bv[KT - 1]) {
-            // from the entry it takes the place of on, the list moves down by one: entries that it
-            // displaces may equal the next ones and keep their order
-            bool take = false;
+          // every entry below cv moves down by one, whatever it equals; no comparison waits for another
 #pragma unroll
-            for (int e = 0; e < KT; e++) {
-              take = take || cv > bv[e];
-              const float tv = bv[e];
-              const int ti = bi[e];
-              bv[e] = take ? cv : bv[e];
-              bi[e] = take ? ci : bi[e];
-              cv = take ? tv : cv;
-              ci = take ? ti : ci;
-            }
+          for (int e = KT - 1; e >= 0; e--) {
+            const bool here = cv > bv[e], above = e > 0 && cv > bv[e > 0 ? e - 1 : 0];
+            bv[e] = above ? bv[e > 0 ? e - 1 : 0] : here ? cv : bv[e];
+            bi[e] = above ? bi[e > 0 ? e - 1 : 0] : here ? ci : bi[e];
           }
         } else {
           int id = class_of(col_id, ci);
