@@ -132,6 +132,9 @@ int hp_tile_cfg_list(hp_tile_cfg* cfgs, int32_t* n);
  * box on the current device, keeps the fastest on the library (as by
  * hp_set_tile_cfg) and returns it in *best (may be NULL).  ms (may be NULL)
  * receives one time per shape in hp_tile_cfg_list order (-1: does not fit).
+ * It is for whole maps: hp_phenotype_map does not divide the ranges of a
+ * library that has a shape, which costs short, ragged and thresholded ranges
+ * up to ten times their time (hp_set_tile_cfg with NULL divides them again).
  * Allocates a stream-ordered scratch map of up to 2^28 ids; synchronises. */
 int hp_autotune(hp_structs* s, hp_tile_cfg* best, float* ms, void* stream);
 
@@ -170,10 +173,13 @@ void hp_batch_plan_free(hp_batch_plan* plan);
 
 /* Ground state of an arbitrary list of sequence ids (e.g. a seeded sample,
  * the paper's sampling mode of Table 3).  Every conformation is scored on the
- * tensor cores (stream-ordered scratch of at most 27 MB, from a pool that keeps 32 MB per library and device), except in small scans (at most 1,024 conformations and n times these at
- * most 2^22), where its table or scratch does not fit, and in calls with both
- * d_cand and d_counters: these run one warp per sequence, with optional exact
- * bound pruning seeded by candidate conformations (the learned proposal).  With A_s(h) = sum_i h_i c_i(s) and B the HH-contact count,
+ * tensor cores (stream-ordered scratch of at most 27 MB, from a pool of the
+ * library that keeps 32 MB per device); candidates make no difference there.
+ * Three kinds of call run one warp per sequence instead: small scans (at most
+ * 1,024 conformations, and n times these at most 2^22), those whose table or
+ * scratch finds no room, and those with both d_cand and d_counters.  They are
+ * pruned by an exact bound, seeded by the candidate conformations (the learned
+ * proposal).  With A_s(h) = sum_i h_i c_i(s) and B the HH-contact count,
  * -E = 10 A + 3 B <= 10 A + 3 min(C, floor(A/2)) (Eq. 1, Table 1 x 10); A
  * depends on a conformation only through its contact-count vector, so the
  * bound is taken once per group of conformations sharing that vector, and a

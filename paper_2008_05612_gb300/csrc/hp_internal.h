@@ -151,9 +151,9 @@ struct PhiTable {
   int log2cap;
 };
 constexpr unsigned kErrPhiFull = 16u;  // error bit: the table is full
-// Eq. 2 numerators of a full 2^N map (robustness tile pass): ADDS to neutral / to_del [S + 1] and
-// counts the -1 genotypes into *negcount (all caller-zeroed); error bits go to *err.  With phi, the
-// same passes also count into the table (S < 65535).
+// Eq. 2 numerators of a full 2^N map (passes over the flips) into neutral / to_del [S + 1], and the count
+// of -1 genotypes into *negcount (all zeroed by the caller); error bits go to *err.  With phi, the same
+// passes also count into the table (S < 65535).
 cudaError_t launch_robustness(const int32_t* d_phen, int N, int S, unsigned long long* neutral,
                               unsigned long long* to_del, unsigned long long* negcount, unsigned* err, cudaStream_t st,
                               const PhiTable* phi = nullptr);

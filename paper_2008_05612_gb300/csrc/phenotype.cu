@@ -146,9 +146,8 @@ struct Cfg {
   // pass 2 reads word j of 32 consecutive records (one per lane): an odd stride in words keeps
   // those loads conflict-free, and the records are written with 4-byte stores.  Where the shared
   // memory has room (tiles of up to 128) its records hold the P tree sums instead of the R - 1 tree
-  // coefficients: a candidate's score is then three reads and two adds instead of 2 + R - 1 reads and R + 1
-  // adds and selects (5x5, where two thirds of
-  // the sequences get here: 2.42 -> 2.14 ms).
+  // coefficients: a candidate's score is then three reads and two adds instead of R + 1 reads and as many
+  // adds and selects (5x5, where two thirds of the sequences get here: 2.42 -> 2.14 ms).
   static constexpr bool kTreeSums = T_ <= 128;
   static constexpr int CS2_RAW = TP_OFF + (kTreeSums ? P : TP_WORDS);
   static constexpr int CS2 = CS2_RAW | 1;
@@ -812,7 +811,8 @@ namespace hp {
 
 // 13 free even residues take the 12-role shape too (two items per odd pattern): a 13-role shape (8 warps,
 // 128 conformations per tile) took 124.1 ms for 2^25 ids of 3x3x3 where this one takes 119.1, 70.5 against 68.2
-// for 2^25 ids of 6x6, and 2.14 against 2.12 for 5x5.
+// for 2^25 ids of 6x6, and 2.14 against 2.12 for 5x5 (whose reversed ids are then written one by one, as
+// where not all of a CTA's even residues are roles).
 // The 11-role shape takes tiles of 128 conformations instead of 64 for libraries of 2^16 or more, where fewer
 // merges per conformation count more than cheaper pass-2 candidates: 2^21 ids of 3x3x3 (103,346
 // conformations) 10.57 -> 8.93 ms, but 2^22 of 6x6 (57,337) 11.46 -> 11.88 and 4x5 (503) 0.19 -> 0.23.

@@ -59,9 +59,8 @@ void default_tile_cfg(int* reg_bits, int* tile);
 // roles: even-pattern bits per CTA (14, or 12 / 11 for the small-role shapes)
 int plan_phenotype(const hp_structs* const* libs, const uint64_t* begins, const uint64_t* counts, int n,
                    int32_t* const* d_phen, int32_t* const* d_aux, int tile, PhenParams& prm, int roles = 14);
-// The compiled shape for blocks with at most max_ne_free free even residues (and libraries of at least
-// min_conf conformations): *roles = 14 (shape
-// unchanged) or 12 / 11 with their own (reg_bits, tile).
+// The compiled shape for blocks with at most max_ne_free free even residues and libraries of at least
+// min_conf conformations: *roles = 14 (shape unchanged) or 12 / 11 with their own (reg_bits, tile).
 void small_roles_shape(int max_ne_free, int min_conf, int* roles, int* reg_bits, int* tile);
 // The role count each entry would get on its own (small_roles_shape of its blocks), into cls.
 int role_classes(const hp_structs* const* libs, const uint64_t* begins, const uint64_t* counts, int n,

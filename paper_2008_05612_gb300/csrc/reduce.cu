@@ -171,18 +171,18 @@ __device__ __forceinline__ unsigned tile_root(const uint16_t* par, unsigned x) {
 
 // ---------------------------------------------------------------- passes over the flips
 
-// Eq. 2 numerators in passes over the map, each reading it once.  A block is 2^13 ids (kRobTileBits)
-// in shared memory: 2^c consecutive ids times every combination of the pass's h bits
-// (c + h = kRobTileBits), the other bits of the id fixed by the block index.  The first pass
-// takes 2^13 consecutive ids and counts the flips of bits 0..12; each later pass counts the flips
-// of its own h bits, so every flip of every genotype is counted once, from shared memory, with
-// the map read 1 + ceil((N - 13) / 8) times instead of once per high bit.  Only genotypes with
+// Eq. 2 numerators in passes over the map, each reading it once.  A block is 2^k ids in shared memory
+// (flip_block_bits: k = 13, 12 for the phi table, less for maps of up to 2^20 ids): 2^c consecutive ids
+// times every combination of the pass's h bits (c + h = k), the other bits of the id fixed by the block
+// index.  The first pass takes 2^k consecutive ids and counts the flips of bits 0..k - 1; each later
+// pass counts the flips of its own h bits, so every flip of every genotype is counted once, from shared
+// memory, with the map read 1 + ceil((N - k) / 8) times instead of once per high bit.  Only genotypes with
 // P(g) >= 0 examine their flips; the -1 row follows from the edge identity
 // sum_{P(g)=-1} #{i: P(g^2^i) = -1} = N N_{-1} - sum_{p>=0} to_del[p].
 // A CTA walks blocks with the next block's asynchronous copy in flight; the block's genotypes
-// that fold are listed first, then examined one per lane.  The counts go to replica blockIdx % R of each phenotype's counters
-// (neutral[r S + p], to_del[r S + p]), so that the atomics of a very designable phenotype are
-// spread over R addresses; robustness_gather adds the replicas up.
+// that fold are listed first, then examined one per lane.  The counts go to replica blockIdx % R of each
+// phenotype's counters (neutral[r S + p], to_del[r S + p]), so that the atomics of a very designable
+// phenotype are spread over R addresses; robustness_gather adds the replicas up.
 struct RobPass {
   int c, h;                   // contiguous low bits of a block; pass bits
   int pos[kRobMaxPassBits];   // positions of the pass bits (all >= c)
@@ -239,11 +239,12 @@ __host__ __device__ constexpr int block_bits(int work) { return work == kPhi ? k
 // shorter loop is faster: 2^25 ids 617 against 639 us.
 template <int WORK, bool SHARE = false>
 __global__ void __launch_bounds__(kRobThreads) flip_pass(const int32_t* __restrict__ phen, int S, const RobPass P,
-                                                               unsigned long long nblocks, int replicas,
-                                                               unsigned long long* __restrict__ neutral_rep,
-                                                               unsigned long long* __restrict__ to_del_rep,
-                                                               unsigned long long* __restrict__ negcount,
-                                                               unsigned* __restrict__ err, const hp::PhiTable phi, int32_t* label) {
+                                                         unsigned long long nblocks, int replicas,
+                                                         unsigned long long* __restrict__ neutral_rep,
+                                                         unsigned long long* __restrict__ to_del_rep,
+                                                         unsigned long long* __restrict__ negcount,
+                                                         unsigned* __restrict__ err, const hp::PhiTable phi,
+                                                         int32_t* label) {
   constexpr bool PHI = WORK == kPhi;
   extern __shared__ int32_t tiles[];  // two blocks, then the list of a block's genotypes that fold
   __shared__ unsigned long long hoff[1 << kRobMaxPassBits];
@@ -259,7 +260,9 @@ __global__ void __launch_bounds__(kRobThreads) flip_pass(const int32_t* __restri
   }
   __syncthreads();
   const int c = P.c;
-  const unsigned cmask = (1u << c) - 1u, ids = 1u << (c + P.h);  // ids < kIds only when N < kRobTileBits
+  const unsigned cmask = (1u << c) - 1u, ids = 1u << (c + P.h);  // at most kIds
+  // Smaller blocks (maps below 2^21 ids) are read word by word: a CTA has one or two of them, so there is
+  // little to overlap, and with a bound on the copies' loop the large maps took 1 to 2 % longer.
   const bool vec = reinterpret_cast<uintptr_t>(phen) % 16 == 0 && c >= 2 && ids == (unsigned)kIds;
   auto block_base = [&](unsigned long long b) {
     unsigned long long base = 0;
@@ -599,13 +602,14 @@ template <class Kernel>
 unsigned pass_grid(Kernel kernel, size_t smem, unsigned long long blocks) {
   if (blocks <= (unsigned long long)sm_count()) return (unsigned)blocks;
   int per_sm = 0;
-  if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kernel, kRobThreads, smem) != cudaSuccess || per_sm < 1) per_sm = 1;
+  if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kernel, kRobThreads, smem) != cudaSuccess || per_sm < 1)
+    per_sm = 1;
   return (unsigned)std::min<unsigned long long>(blocks, (unsigned long long)sm_count() * per_sm);
 }
 
-// log2 of the ids per block: `most`, or less for small maps, so that they still have 2^7 blocks or so to spread over
-// the SMs and one later pass (4x4, 2^16 ids: Eq. 2 passes 20 -> 12 us,
-// networks 41 + 25 -> 10 + 18 us, against blocks of 2^13).
+// log2 of the ids per block: `most`, or less for small maps, so that they still have 2^7 blocks or so to
+// spread over the SMs and one later pass (4x4, 2^16 ids: Eq. 2 passes 20 -> 12 us, networks 41 + 25 ->
+// 10 + 18 us, against blocks of 2^13).
 int flip_block_bits(int N, int most) { return std::min(N, std::max(9, std::min(most, N - 8))); }
 
 // The passes over the flips of an N-bit map: bits [0, k) first, then the high bits [k, N) in
@@ -660,8 +664,8 @@ cudaError_t launch_robustness(const int32_t* d_phen, int N, int S, unsigned long
   }
   for (const RobPass& p : plan) {
     if (rep)
-      pass<<<grid, kRobThreads, smem, st>>>(d_phen, S, p, blocks, kRobReplicas, rep, rep + (size_t)kRobReplicas * S, negcount,
-                                            err, table, nullptr);
+      pass<<<grid, kRobThreads, smem, st>>>(d_phen, S, p, blocks, kRobReplicas, rep, rep + (size_t)kRobReplicas * S,
+                                            negcount, err, table, nullptr);
     else
       pass<<<grid, kRobThreads, smem, st>>>(d_phen, S, p, blocks, 1, neutral, to_del, negcount, err, table, nullptr);
   }
@@ -700,8 +704,8 @@ extern "C" int hp_neutral_components(const int32_t* d_phen, int32_t N, int32_t S
     for (const RobPass& p : hp::flip_passes(N, kRobTileBits)) {
       const auto pass = p.first ? first : later;
       const size_t bytes = p.first ? smem1 : smem;
-      pass<<<hp::pass_grid(pass, bytes, blocks), kRobThreads, bytes, st>>>(d_phen, S, p, blocks, 1, nullptr, nullptr, nullptr,
-                                                                          err, hp::PhiTable{}, d_label);
+      pass<<<hp::pass_grid(pass, bytes, blocks), kRobThreads, bytes, st>>>(d_phen, S, p, blocks, 1, nullptr, nullptr,
+                                                                          nullptr, err, hp::PhiTable{}, d_label);
     }
     const unsigned grid = (unsigned)std::min<unsigned long long>((total + 1023) / 1024, (unsigned long long)sm_count() * 16);
     cc_finish<<<grid, 256, 0, st>>>(d_phen, total, d_label, reinterpret_cast<unsigned long long*>(d_ncomp));

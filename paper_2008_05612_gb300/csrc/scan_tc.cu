@@ -12,8 +12,8 @@
 // scan_tc_kernel: persistent CTAs, one per SM, each a contiguous run of (256-sequence block,
 // 256-conformation tile) units.  The block's features (2 x 128 rows) are written to shared memory by
 // the epilogue warps; the conformations stream through a ring of stages of 8 KB slabs (256
-// conformations x 32 pairs, stored in the order the tensor core reads them; one cp.async.bulk a stage).  Both halves of
-// the block use a slab while it is resident, which halves the L2 traffic per multiplication to
+// conformations x 32 pairs, stored in the order the tensor core reads them; one cp.async.bulk a stage).
+// Both halves of the block use a slab while it is resident, which halves the L2 traffic per multiplication to
 // 32 B/clk/SM (one half alone would need 64, more than L2 delivers to all SMs at once); while the
 // tensor core works on one half's accumulator (256 TMEM columns) the epilogue drains the other's.
 // The epilogue keeps per sequence the best score, the second best over groups of 32
@@ -21,8 +21,8 @@
 // three-input maxima and five more instructions per 32 scores.
 // A unit takes 2 x 128 clk per 32 pairs at the tensor cores' rate; each half has one accumulator, so a
 // half's drain and hand-over (about 400 clk) overlap only the other half's multiplications.
-// Measured (call, ids in L2): 16,384 ids of 3x3x3 170 us, the warp scan 13,600 us; 65,536 ids of 6x6
-// 660 us, the pruned warp scan 6,400 us; floors at 128 clk per 128 x 256 x 32: 110 and 480 us.
+// Measured (call, ids in L2): 16,384 ids of 3x3x3 160 us, the warp scan 13,600 us; 65,536 ids of 6x6
+// 648 us, the pruned warp scan 6,600 us; floors at 128 clk per 128 x 256 x 32: 110 and 480 us.
 //
 // scan_tc_resolve: one warp per sequence merges the runs' results and scores the one group of 32
 // conformations exactly, which gives the lowest minimiser, the tie and the energy gap.
@@ -62,7 +62,8 @@ constexpr uint32_t kF13 = 0x55, kFm10 = 0xD2, kF1 = 0x38, kF448 = 0x7E;
 
 struct TcParams {
   const uint8_t* tab;              // ntiles x nk slabs of kSlabB bytes
-  const uint16_t* pairs;           // 32 nk entries: even index | odd index << 8; 0xFFFF constant, 0xFFFE unused
+  const uint16_t* pairs;           // 32 nk entries: even index | odd index << 8; 0x1F1F (bits that are always
+                                   // clear) for the constant and the unused columns
   const unsigned long long* ids;   // n ids, or NULL: base + row
   unsigned long long base;
   long long n, units;
@@ -257,8 +258,9 @@ __global__ void __launch_bounds__(kThreads, 1) scan_tc_kernel(const TcParams p) 
     // ---------------------------------------------------------------- MMA issuers, one per half
     // A wait on a barrier that is already complete costs the issuing warp about 200 clk, more than the
     // tensor core has queued; with an issuer per half one half's MMAs run during the other's waits
-    // (one issuer for both halves: 999 instead of 723 us per 65,536 ids of 3x3x3).  The whole warp walks the loop and one
-    // elected lane issues, so that addresses and descriptors stay in uniform registers.
+    // (one issuer for both halves: 999 instead of 723 us per 65,536 ids of 3x3x3 with the waits and stages
+    // as they then were; 573 now).  The whole warp walks the loop and one elected lane issues, so that
+    // addresses and descriptors stay in uniform registers.
     const int h = warp - 1;
     int slot = 0;
     uint32_t round = 0, seg = 0, uses = 0;
@@ -668,7 +670,7 @@ int scan_tc(const hp_structs* s, const ScanTc& a, cudaStream_t st, long long* do
   // The largest stage (slabs per wait, copy and commit) that leaves one stage beside the tile's, which
   // stay resident for both halves.  Every stage costs the issuers a wait and a commit: 65,536 ids of
   // 6x6 (10 slabs) took 925 us with stages of 2 slabs, 812 with 3 and 700 with 5; 3x3x3 (5 slabs)
-  // 1464 us with 1, 878 with 3 and 627 with 5.
+  // 1464 us with 1, 878 with 3 and 627 with 5 (before other changes: 648 and 573 us now).
   for (p.cs = std::min(p.nk, kMaxStage); p.cs >= 1; p.cs--) {
     p.nslots = std::min(kMaxSlots, (kSmemMax - 128 - abytes) / (p.cs * kSlabB));
     if (p.nslots > (p.nk + p.cs - 1) / p.cs) break;

@@ -7,8 +7,8 @@
 //   warp 1            MMA issuer: four tcgen05.mma (M 128, N 256, K 16) per chunk into one of two
 //                     tensor-memory accumulators (2 x 256 columns), commit -> empty[s] frees the
 //                     stage, commit -> tmem_full[a] hands the finished accumulator over;
-//   warps 2..9        epilogue, two warps per lane quarter and 128 columns each: tcgen05.ld
-//                     (warp w reads lanes 32 (w % 4) .. +31 = tile rows), bias, ReLU, stores
+//   warps 2..         epilogue, 16 warps (64 columns each, four per lane quarter) or, in top-k mode, 8 (128
+//                     columns): tcgen05.ld (warp w reads lanes 32 (w % 4) .. +31 = tile rows), bias, ReLU, stores
 //                     through a padded shared-memory square (coalesced rows), a per-row
 //                     running top-k, or the softmax statistics or gradient (the gradient's
 //                     32 x 32 blocks leave through TMA stores); then arrive on tmem_empty[a].
@@ -446,8 +446,9 @@ __global__ void __launch_bounds__(Shape<KT>::kThreads, 1)
     // Every instruction here delays the next MMA (the tensor core has few queued, and the epilogue warps
     // compete for the issue slots), so the loop is kept short: the whole warp walks it and one elected
     // lane issues (no loops over divergent lanes, operands in uniform registers), a wait is one poll
-    // where the barrier is complete (looking a chunk ahead did not help), and descriptors are one word.  Proposal top-4 of 16,384
-    // ids 818 -> 776 us, training step 979 -> 950 us against a single lane in a divergent branch.
+    // where the barrier is complete (looking a chunk ahead did not help), and descriptors are one word.
+    // Proposal top-4 of 16,384 ids 818 -> 776 us, training step 979 -> 950 us against a single lane in a
+    // divergent branch.
     uint32_t s = 0, par = 0, it = 0, tl = 0;  // stage and its round's parity, chunks, tiles
     bool ok = true;
     const uint32_t idesc = IDESC | ((uint32_t)(p.a_mn != 0) << 15) | ((uint32_t)(p.b_mn != 0) << 16);
