@@ -17,8 +17,8 @@
 // of its columns (at most 65,536 bits) in shared memory.  The -1 column is always a row's last entry, and
 // the -1 row's entries follow from a scan over the phenotypes.  Nothing waits for the host until the end.
 // The map of 2^25 ids at the 3x3x3 folding density (0.9 million entries) took 5.41 ms with a second pass
-// over the map for the table and a bitonic sort of all entries (210 launches); now 0.61 ms, of which the
-// passes over the map are 0.41.
+// over the map for the table and a bitonic sort of all entries (210 launches); now 0.63 ms, of which the
+// passes over the map are 0.40.
 #include <cuda_runtime.h>
 
 #include <algorithm>

@@ -222,7 +222,7 @@ __device__ __forceinline__ void phi_add(const hp::PhiTable& t, uint32_t key, uns
 // phenotype); or the unions of the neutral networks.  For the networks the first pass joins each block of
 // 2^13 ids by a union-find in shared memory and writes the block's labels (-1 where the id does not fold),
 // and the later passes join ids across the pass's bits through the labels in global memory, comparing
-// phenotypes in shared memory.  2^25 ids at the 3x3x3 density: 200 + 286 us and 84 us for the last walk (the
+// phenotypes in shared memory.  2^25 ids at the 3x3x3 density: 190 + 285 us and 98 us for the last walk (the
 // unions wait on dependent reads), where one pass that read every partner from global memory and joined
 // all flips through global labels took 67 + 566 + 178 us.
 enum FlipWork { kRobustness, kPhi, kJoinFirst, kJoin };
